@@ -1,0 +1,58 @@
+"""The training kernel's tiles: gradients at batches around the tile sizes and the
+block count against the float64 chain rule, and the same bits on every run."""
+import numpy as np
+import pytest
+
+from oracle import screener as osc
+from workloads import data
+
+from parity import car_env, gpu_model
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def setup():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1906_02318_gb300 import build, mpmi
+    build.build()
+    ctx = mpmi.Context(0)
+    return mpmi, ctx, gpu_model(mpmi, ctx, car_env())
+
+
+# tiles of 16 samples up to 16 per SM (152 SMs: 2432), 32 up to 4864, then 64; more
+# tiles than blocks past 64 per SM (9728).  exact: max_batch = the batch, which
+# bounds the blocks to one per 32 samples
+@pytest.mark.parametrize("B, exact", [(1, True), (15, True), (16, False), (17, True), (33, True),
+                                      (250, True), (250, False), (2433, False), (4864, True),
+                                      (4865, False), (8192, False), (9729, False), (20011, True)])
+def test_gradients_around_the_tiles(setup, B, exact):
+    import torch
+    lib, ctx, model = setup
+    w = data.screener_init(7)
+    rng = np.random.default_rng(B)
+    f = data.to_f32_exact(rng.uniform(-1, 1, (B, 12)))
+    t = data.to_f32_exact(rng.uniform(0, 1, B))
+    scr = lib.Screener(ctx, model, w, max_batch=B if exact else 24000, max_slots=64)
+    fd = torch.tensor(f, dtype=torch.float32, device="cuda")
+    td = torch.tensor(t, dtype=torch.float32, device="cuda")
+    out = []
+    for _ in range(2):
+        g = torch.full((lib.SCREENER_PARAMS,), float("nan"), device="cuda")
+        loss = torch.full((1,), float("nan"), device="cuda")
+        scr.gradients(fd, td, g, loss)
+        torch.cuda.synchronize()
+        out.append((g.cpu().numpy(), float(loss.item())))
+    scr.free()
+    assert np.array_equal(out[0][0], out[1][0]) and out[0][1] == out[1][1]
+    cache = osc.forward(w, f)
+    ref = osc.backward(w, cache, t)
+    got = lib.unpack_weights(out[0][0])
+    assert out[0][1] == pytest.approx(osc.loss(cache["y"], t), rel=1e-5)
+    for k in ref:
+        # float32 sums of products: the error of each is a few hundred roundings
+        # (2^-24) of the largest entry's terms
+        scale = float(np.max(np.abs(ref[k])))
+        assert np.max(np.abs(np.asarray(got[k]) - ref[k])) <= 1e-4 * scale + 1e-9, k
