@@ -369,7 +369,10 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_tick_kernel(const __grid_con
       // candidates test step t
       bool ok = box_ok<NX>(a.safety, z);
       if constexpr (B::TRACK) {
-        if (track_on) ok = ok && track_ok<1>(a.safety.track, tv, z[0], z[1], 0, alive && ok);
+        if (track_on) {  // uniform; every lane of the warp takes part
+          const bool on_road = track_ok_warp(a.safety.track, tv, z[0], z[1], alive && ok);
+          ok = ok && on_road;
+        }
       }
       if (alive) {
         if (ok) ttv = t;
