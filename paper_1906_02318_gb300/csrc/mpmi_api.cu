@@ -57,7 +57,8 @@ static TickKernel pick_tick(int kind, int lanes, int cands, bool traj, bool nois
 // H = 60, CUDA events, L2 flushed): N = 1024 16 lanes 28 us; N = 4096 8 lanes
 // 38 us against 47 (2 lanes) and 69 (1 lane); N = 8192 2 lanes 47 us against 62
 // (8 lanes) and 69; N = 16384 2 lanes 60 us against 69 (1 lane); N = 32768 1 lane
-// 103 us against 110 (2 lanes); from ~48k slots two candidates per thread.  The
+// 103 us against 110 (2 lanes); past eight tiles per SM (38,912 slots) two candidates
+// per thread (N = 40000 124 us against 131).  The
 // two-lane shape keeps two warps per SM sub-partition while they fit one wave
 // (two 128-thread blocks per SM), hiding each other's latency.  Balance bot
 // N <= 4096 with 4 lanes 12.6 against 13.4..14.1 us, else one lane.  Blocks of
@@ -66,16 +67,30 @@ static TickKernel pick_tick(int kind, int lanes, int cands, bool traj, bool nois
 // blocks stage K and the track grid fewer times.
 constexpr int kDefaultBlock = 128;
 
+// Whether a one-lane launch over n slots takes sorted units, where one wave of warps
+// holds `wave` slots.  With more than ~1.6 tiles per warp the tiles a warp saves by
+// sorting outweigh drawing every candidate twice (balance bot N = 65536, 1.7 tiles,
+// 20.8 -> 18.8 us); below, the last round's few tiles run alone either way (race car
+// N = 100000, 1.3 tiles, 217 us unsorted, 225 sorted).  The race car also gains where
+// every tile has a warp of its own (N = 24000 87.7 -> 84.3 us, N = 65536 150 -> 145 us):
+// its warps share the shared-memory pipe, which tiles that leave early free.
+static bool units_pay(int kind, long long n, long long wave) {
+  if (10 * n >= 16 * wave) return true;
+  return kind == kCar && 2 * n >= wave && n <= wave;
+}
+
 // Threads per block the library picks for a shape.  The race car's one-lane
 // shapes: where the warp-tiles fit one block of at most eight warps per SM,
 // blocks of ceil(tiles / SMs) warps, one per SM, load the SMs more evenly than
 // two four-warp blocks on some SMs and one on the rest (measured 4-10 % faster
 // from 20k to 76k slots); everything else kDefaultBlock.
 static int default_block(int kind, int lanes, int cands, long long n_slots, int sms) {
-  if (kind == kCar && lanes == 1) {
+  if (lanes == 1) {
     const long long tiles = (n_slots + 32LL * cands - 1) / (32LL * cands);
     const long long w = (tiles + sms - 1) / sms;
-    if (w > 4 && w <= kMaxBlock / 32) return (int)(32 * w);
+    if (kind == kCar && w > 4 && w <= kMaxBlock / 32) return (int)(32 * w);
+    // sorted units: one queue of tiles per SM, eight warps on it
+    if (units_pay(kind, n_slots, 256LL * cands * sms) && w > kMaxBlock / 32) return kMaxBlock;
   }
   return kDefaultBlock;
 }
@@ -89,7 +104,7 @@ static void default_shape(int kind, int n_slots, int sms, int* lanes, int* cands
     else if (n <= (long long)sms * 128) *lanes = 2;       // two-lane warps fit one wave
     else {
       *lanes = 1;
-      *cands = n > 48 * 1024 ? 2 : 1;
+      *cands = n > 256LL * sms ? 2 : 1;  // past one tile for each of an SM's eight warps
     }
   } else {
     *lanes = (kind == kBot && (long long)n_slots * 4 <= (long long)sms * 128) ? 4 : 1;
@@ -306,27 +321,46 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
   if (!k.fn) return fail(MPMI_E_UNSUPPORTED, "tick kernel not compiled for this launch shape");
   const size_t smem = k.k_smem + (a.safety.has_track ? (size_t)a.safety.track.blob_bytes : 0);
   const int t = (traj ? 1 : 0) + (small ? 2 : 0) + (noise ? 4 : 0) + (small && lanes == 16 ? 8 : 0);
+  const int per_warp = 32 / lanes * cands;
+  const int n_work = (n_hint > 0 && n_hint < s->n_slots) ? n_hint : s->n_slots;
   if (s->max_grid[t] == 0 || s->grid_smem[t] != smem) {
-    // static (lane exchange) plus dynamic shared memory may pass the 48 KB default
-    if (smem > 0) {
-      cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(k.k_smem + kMaxTrackBytes));
-      if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
-    }
     int nb = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn, block, smem);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-    if (nb < 1) return fail(MPMI_E_UNSUPPORTED, "tick kernel cannot be resident with this block");
+    s->unit[t] = 0;
+    if (k.fn_units && a.slot_list == nullptr) {
+      const size_t most = smem + unit_bytes(kUnitMax);
+      cudaError_t e =
+          cudaFuncSetAttribute(k.fn_units, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)(k.k_smem + kMaxTrackBytes + unit_bytes(kUnitMax)));
+      if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn_units, block, most);
+      if (e != cudaSuccess) return cuda_fail(e, "sorted units: function attributes");
+      const long long blocks = (long long)nb * s->ctx->sm_count;
+      if (nb > 0 && units_pay(s->model->kind, n_work, blocks * (block / 32) * per_warp)) {
+        // equal shares of the slots per block, in as few rounds as kUnitMax allows
+        const long long rounds = (n_work + blocks * kUnitMax - 1) / (blocks * kUnitMax);
+        s->unit[t] = (int)((n_work + blocks * rounds - 1) / (blocks * rounds));
+      }
+    }
+    if (s->unit[t] == 0) {
+      // static (lane exchange) plus dynamic shared memory may pass the 48 KB default
+      if (smem > 0) {
+        cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)(k.k_smem + kMaxTrackBytes));
+        if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+      }
+      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn, block, smem);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+      if (nb < 1) return fail(MPMI_E_UNSUPPORTED, "tick kernel cannot be resident with this block");
+    }
     s->max_grid[t] = nb * s->ctx->sm_count;
     s->grid_smem[t] = smem;
   }
-  const int wpb = block / 32;
-  const int per_warp = 32 / lanes * cands;
-  const int n_work = (n_hint > 0 && n_hint < s->n_slots) ? n_hint : s->n_slots;
-  const int n_wtiles = (n_work + per_warp - 1) / per_warp;
-  int grid = (n_wtiles + wpb - 1) / wpb;
+  a.unit = s->unit[t];
+  const int per_block = a.unit > 0 ? a.unit : per_warp * (block / 32);
+  int grid = (n_work + per_block - 1) / per_block;
   if (grid > s->max_grid[t]) grid = s->max_grid[t];
-  k.launch(a, grid, block, smem, st);
+  if (a.unit > 0) k.launch_units(a, grid, block, smem + unit_bytes(a.unit), st);
+  else k.launch(a, grid, block, smem, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "tick kernel launch");
   return MPMI_OK;

@@ -15,15 +15,18 @@ struct TickKernel {
   const void* fn = nullptr;
   void (*launch)(const TickArgs&, int, int, size_t, cudaStream_t) = nullptr;
   size_t k_smem = 0;  // bytes of K staged in shared memory
+  // the same shape over sorted units (one lane, no trajectories)
+  const void* fn_units = nullptr;
+  void (*launch_units)(const TickArgs&, int, int, size_t, cudaStream_t) = nullptr;
 };
 
 // A TickArgs with `chained` set is launched with programmatic stream
 // serialisation (it may start before the previous kernel on the stream ends and
 // waits for it in the kernel); any other launch is an ordinary one.
-template <int KIND, int L, int C, bool KSMEM, bool TRAJ, bool NOISE>
+template <int KIND, int L, int C, bool KSMEM, bool TRAJ, bool NOISE, bool UNITS>
 static void launch_tick(const TickArgs& a, int grid, int block, size_t smem, cudaStream_t st) {
   if (!a.chained) {
-    tick_kernel<KIND, L, C, KSMEM, TRAJ, false, NOISE><<<grid, block, smem, st>>>(a);
+    tick_kernel<KIND, L, C, KSMEM, TRAJ, false, NOISE, UNITS><<<grid, block, smem, st>>>(a);
     return;
   }
   cudaLaunchConfig_t cfg = {};
@@ -36,14 +39,19 @@ static void launch_tick(const TickArgs& a, int grid, int block, size_t smem, cud
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, tick_kernel<KIND, L, C, KSMEM, TRAJ, false, NOISE>, a);
+  cudaLaunchKernelEx(&cfg, tick_kernel<KIND, L, C, KSMEM, TRAJ, false, NOISE, UNITS>, a);
 }
 
 template <int KIND, int L, int C, bool KSMEM, bool TRAJ, bool NOISE>
 static TickKernel make_kernel() {
   TickKernel k;
   k.fn = reinterpret_cast<const void*>(&tick_kernel<KIND, L, C, KSMEM, TRAJ, false, NOISE>);
-  k.launch = &launch_tick<KIND, L, C, KSMEM, TRAJ, NOISE>;
+  k.launch = &launch_tick<KIND, L, C, KSMEM, TRAJ, NOISE, false>;
+  if constexpr (L == 1 && !TRAJ) {
+    k.fn_units =
+        reinterpret_cast<const void*>(&tick_kernel<KIND, L, C, KSMEM, TRAJ, false, NOISE, true>);
+    k.launch_units = &launch_tick<KIND, L, C, KSMEM, TRAJ, NOISE, true>;
+  }
   k.k_smem = (size_t)ksmem_words<KIND, L, KSMEM, true>() * 16;
   return k;
 }

@@ -611,7 +611,8 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
                                          const float* xs, const float* uh, float sn, float cs,
                                          const KR& kr, const float4* sK4, const TrackView& tv,
                                          float* xbuf, unsigned long long& best,
-                                         unsigned int& n_safe, unsigned int& n_exec) {
+                                         unsigned int& n_safe, unsigned int& n_exec,
+                                         const uint16_t* order = nullptr, int base = 0) {
   using B = BasisTraits<KIND>;
   constexpr int N = B::N, NX = B::NX, NU = B::NU, NP = B::NP;
   constexpr int R = N / L;
@@ -633,8 +634,13 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
   float* traj[C];
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    const int pos = wt * PER_WARP + c * GPW + g;
+    int pos = wt * PER_WARP + c * GPW + g;
     valid[c] = pos < n_eval;
+    if constexpr (L == 1) {
+      // a tile of a sorted unit (sort_unit): position pos of the unit is slot
+      // base + order[pos]
+      if (order != nullptr && valid[c]) pos = base + (int)order[pos];
+    }
     slot[c] = (valid[c] && a.slot_list) ? a.slot_list[pos] : pos;
     float xi[NU];
     if (valid[c]) {
@@ -976,6 +982,77 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
   }
 }
 
+// ---- sorted units (one-lane shapes) ----
+// A warp's candidates leave at different steps, and a warp runs until its last one
+// leaves: with candidates drawn at random nearly every warp runs the whole horizon,
+// and 11 (race car, H = 60) to 60 % (balance bot, H = 100) of its lane-steps are
+// idle.  A candidate's time to violation follows its first input closely, so a block
+// that has several tiles per warp takes its slots as units of up to kUnitMax, orders
+// a unit by the first input (a counting sort over kUnitBins bins of the input box)
+// and lets its warps take the unit's tiles from a counter: a tile's candidates then
+// leave together, and warps that the scheduler favours take more tiles.  The order
+// changes no result (a minimum, integer sums, per-slot outputs).
+// GB300, ticks back to back: balance bot H = 50, N = 1048576 207 -> 164 us, H = 100,
+// N = 200000 86 -> 44 us; race car H = 60, N = 65536 150 -> 145 us, N = 262144 578 ->
+// 460 us, H = 100, N = 131072 518 -> 322 us.
+constexpr int kUnitMax = 8192, kUnitBins = 256;
+
+// Shared-memory bytes of a unit: bin counters, each candidate's place and bin.
+MPMI_HD constexpr size_t unit_bytes(int unit) {
+  return 4 * kUnitBins + (3 * (size_t)unit + 15) / 16 * 16;
+}
+
+// Orders positions 0 .. cnt - 1 (slots base + position) by bins of the first input and
+// restarts the tile counter (whole block; buf: unit_bytes(unit) of shared memory).
+template <int NU, class P>
+__device__ __forceinline__ const uint16_t* sort_unit(const P& a, TickDyn d, int base, int cnt,
+                                                     int unit, const float* uh, char* buf,
+                                                     int* next) {
+  uint32_t* bins = reinterpret_cast<uint32_t*>(buf);
+  uint16_t* order = reinterpret_cast<uint16_t*>(bins + kUnitBins);
+  uint8_t* bin = reinterpret_cast<uint8_t*>(order + unit);
+  const int tid = threadIdx.x;
+  const float scale = (float)kUnitBins / a.in_w[0];
+  __syncthreads();  // every warp is done with the previous unit
+  if (tid == 0) *next = 0;
+  for (int b = tid; b < kUnitBins; b += blockDim.x) bins[b] = 0;
+  __syncthreads();
+  for (int i = tid; i < cnt; i += blockDim.x) {
+    float xi[NU];
+    candidate_value<NU>(a, d.t_lo, d.t_hi, base + i, uh, xi);
+    // out-of-box and NaN inputs land in an end bin
+    const float f = fminf(fmaxf((xi[0] - a.in_lo[0]) * scale, 0.f), (float)(kUnitBins - 1));
+    bin[i] = (uint8_t)f;
+    atomicAdd(&bins[(int)f], 1u);
+  }
+  __syncthreads();
+  if (tid < 32) {  // exclusive prefix: eight bins per lane
+    constexpr int PER = kUnitBins / 32;
+    uint32_t n[PER], sum = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      n[j] = bins[tid * PER + j];
+      sum += n[j];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(kFull, incl, o);
+      if (tid >= o) incl += v;
+    }
+    uint32_t at = incl - sum;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      bins[tid * PER + j] = at;
+      at += n[j];
+    }
+  }
+  __syncthreads();
+  for (int i = tid; i < cnt; i += blockDim.x) order[atomicAdd(&bins[bin[i]], 1u)] = (uint16_t)i;
+  __syncthreads();
+  return order;
+}
+
 // End of a tick launch: warp -> block -> grid reduction of the selection key
 // and the counts into the session's reduction record (one atomicMin/atomicAdd per
 // block); the block that finishes last decodes the result and resets the record.
@@ -1054,9 +1131,11 @@ __device__ __forceinline__ void session_epilogue(const P& a, unsigned long long 
 //   PARTIALS no-allocation variant: each block stores its partial (key,
 //            counts) in a.partials and the last block folds them, instead of
 //            atomics on a session's reduction record;
-//   NOISE    add Alg. 2's Gaussian noise z_i after every prediction step.
+//   NOISE    add Alg. 2's Gaussian noise z_i after every prediction step;
+//   UNITS    blocks take sorted units of a.unit slots (one lane; an instance of its
+//            own, since the two-lane kernel ran 7 % slower with this path compiled in).
 template <int KIND, int L, int C, bool KSMEM, bool TRAJ, bool PARTIALS = false,
-          bool NOISE = false>
+          bool NOISE = false, bool UNITS = false>
 __global__ void __launch_bounds__(kMaxBlock) tick_kernel(const __grid_constant__ TickArgs a) {
   using B = BasisTraits<KIND>;
   constexpr int N = B::N, NX = B::NX, NU = B::NU;
@@ -1076,7 +1155,7 @@ __global__ void __launch_bounds__(kMaxBlock) tick_kernel(const __grid_constant__
   __shared__ __align__(16) float s_x[(L > 1) ? NW : 1][2][GPW][S];
   __shared__ unsigned long long s_key[NW];
   __shared__ unsigned long long s_cnt[NW];
-  __shared__ int s_last;
+  __shared__ int s_last, s_next;  // s_next: the unit's next tile (UNITS)
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int q = lane % L;
@@ -1107,7 +1186,8 @@ __global__ void __launch_bounds__(kMaxBlock) tick_kernel(const __grid_constant__
     const int wpb0 = blockDim.x >> 5;
     const long long tiles = ((long long)n_eval + GPW * C - 1) / (GPW * C);
     const long long need = (tiles + wpb0 - 1) / wpb0;
-    n_active = (unsigned int)(need < 1 ? 1 : (need < (long long)gridDim.x ? need : gridDim.x));
+    if constexpr (!UNITS)  // a launch over sorted units has no block too many
+      n_active = (unsigned int)(need < 1 ? 1 : (need < (long long)gridDim.x ? need : gridDim.x));
     if (blockIdx.x >= n_active) return;
   }
 
@@ -1189,10 +1269,31 @@ __global__ void __launch_bounds__(kMaxBlock) tick_kernel(const __grid_constant__
   unsigned int n_safe = 0, n_exec = 0;
   const int wpb = blockDim.x >> 5;
   constexpr int PER_WARP = GPW * C;  // candidate slots per warp-tile
-  const int n_wtiles = failed ? 0 : (n_eval + PER_WARP - 1) / PER_WARP;
-  for (int wt = blockIdx.x * wpb + warp; wt < n_wtiles; wt += gridDim.x * wpb)
-    run_tile<KIND, L, C, KSMEM, TRAJ, NOISE, !PARTIALS>(a, dyn_of(a), a.safety, wt, n_eval, xs, uh, sn, cs, kr, sK4, tv,
-                                      &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec);
+  const auto tile = [&](int wt, int cnt, const uint16_t* order, int base) {
+    run_tile<KIND, L, C, KSMEM, TRAJ, NOISE, !PARTIALS>(
+        a, dyn_of(a), a.safety, wt, cnt, xs, uh, sn, cs, kr, sK4, tv,
+        &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec, order, base);
+  };
+  if constexpr (UNITS) {
+    char* buf = reinterpret_cast<char*>(s_dyn + KWORDS) +
+                (track_on ? a.safety.track.blob_bytes : 0);
+    for (int base = failed ? n_eval : (int)blockIdx.x * a.unit; base < n_eval;
+         base += (int)gridDim.x * a.unit) {
+      const int cnt = min(a.unit, n_eval - base);
+      const uint16_t* order = sort_unit<NU>(a, dyn_of(a), base, cnt, a.unit, uh, buf, &s_next);
+      while (true) {
+        int wt = 0;
+        if (lane == 0) wt = atomicAdd(&s_next, 1);
+        wt = __shfl_sync(kFull, wt, 0);
+        if (wt * PER_WARP >= cnt) break;
+        tile(wt, cnt, order, base);
+      }
+    }
+  } else {
+    const int n_wtiles = failed ? 0 : (n_eval + PER_WARP - 1) / PER_WARP;
+    for (int wt = blockIdx.x * wpb + warp; wt < n_wtiles; wt += gridDim.x * wpb)
+      tile(wt, n_eval, nullptr, 0);
+  }
 
   if constexpr (!PARTIALS) {
     session_epilogue<NU>(a, best, n_safe, n_exec, uh, failed, n_active);

@@ -1,0 +1,80 @@
+"""Ticks over sorted units (one lane per candidate, many candidates) against the same
+ticks in a shape that never sorts, bit for bit in every per-slot output."""
+import numpy as np
+import pytest
+
+from workloads import data
+
+from parity import bot_env, car_env, gpu_model, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def setup():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1906_02318_gb300 import build, mpmi
+    build.build()
+    ctx = mpmi.Context(0)
+    envs = dict(bot=bot_env(), car=car_env())
+    return mpmi, ctx, {k: (e, gpu_model(mpmi, ctx, e)) for k, e in envs.items()}
+
+
+def _same(a, b):
+    assert np.array_equal(a["ttv"], b["ttv"]) and np.array_equal(a["cost"], b["cost"],
+                                                                equal_nan=True)
+    for k in ("index", "status", "n_safe", "ttv", "executed_steps", "n_slots"):
+        assert a["result"][k] == b["result"][k]
+    assert np.array_equal(a["result"]["u_r"], b["result"]["u_r"])
+
+
+# one tile per warp (race car), several tiles per warp, two units per block (a unit
+# holds 8192 slots: more than 152 x 8192 of them), ragged ends; with and without u_h,
+# the grid sampler, per-step noise, two candidates per thread
+@pytest.mark.parametrize("which,N,H,kw", [
+    ("car", 20001, 60, {}), ("car", 38911, 30, {}), ("car", 38912, 60, {}),
+    ("car", 65536, 60, {}), ("car", 150001, 30, {"include_user": False}),
+    ("car", 130321, 25, {"sampler": "grid"}), ("car", 140000, 20, {"noise": True}),
+    ("bot", 62500, 50, {}), ("bot", 70001, 50, {"include_user": False}),
+    ("bot", 131072, 100, {"sampler": "grid"}), ("bot", 100003, 30, {"noise": True}),
+    ("bot", 100003, 30, {"cands": 2}), ("bot", 1300001, 20, {})])
+def test_sorted_units_change_no_result(setup, which, N, H, kw):
+    lib, ctx, envs = setup
+    env, model = envs[which]
+    kw = dict(kw)
+    noise, cands = kw.pop("noise", False), kw.pop("cands", 0)
+    x_t = (np.array([0.1, 0.3, -0.5, 0.4]) if which == "bot" else
+           data.car_start_state(env.track, vx=13.0) + np.array([1.0, -0.5, 0.05, 0, 0, 0]))
+    u_h = data.to_f32_exact(data.user_input_once(5, env.lo, env.hi))
+    out = []
+    for shape in (dict(cands=cands, lanes=1 if cands else 0), dict(lanes=2)):
+        s = lib.Session(ctx, model, N, H, env.lo, env.hi, seed=9, **kw, **shape)
+        if noise:
+            s.set_noise([0.002] * env.spec.lo.size)
+        out.append([run_gpu(lib, s, x_t, u_h, tick=t) for t in (0, 1 << 33)])
+        s.close()
+    for a, b in zip(*out):
+        _same(a, b)
+
+
+@pytest.mark.parametrize("which", ["bot", "car"])
+def test_caller_samples_outside_the_box(setup, which):
+    """Caller samples may lie anywhere: outside the box, infinite, NaN."""
+    import torch
+    lib, ctx, envs = setup
+    env, model = envs[which]
+    N = 140003
+    rng = np.random.default_rng(3)
+    c = rng.uniform(3 * env.lo, 3 * env.hi, size=(N, len(env.lo))).astype(np.float32)
+    c[::97, 0], c[5::101, 0], c[7::103, 0] = np.nan, np.inf, -np.inf
+    cd = torch.tensor(c, device="cuda")
+    x_t = np.zeros(4) if which == "bot" else data.car_start_state(env.track, vx=13.0)
+    u_h = data.to_f32_exact(data.user_input_once(6, env.lo, env.hi))
+    out = []
+    for lanes in (0, 2):
+        s = lib.Session(ctx, model, N, 20, env.lo, env.hi, sampler="external", lanes=lanes)
+        out.append(run_gpu(lib, s, x_t, u_h, candidates=cd))
+        s.close()
+    _same(*out)
