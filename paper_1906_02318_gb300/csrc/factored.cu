@@ -16,13 +16,17 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "internal.h"
 #include "tick_kernel.cuh"
 
 namespace mpmi {
 
-constexpr int kFactBlock = 128;
-constexpr int kFactCands = 8;  // candidates per warp-tile (lanes 0..7 draw them)
+// Most threads of a block.  One block per SM stages the track grid and builds V once
+// for all of its warps (64 registers each); five blocks of 128 threads did both five
+// times per SM.
+constexpr int kFactBlock = 1024;
 
 // Rows P_t = C K^t, t = 1..H: P_1 is the first NX rows of K and P_t = P_{t-1} K
 // (each entry one FMA chain over i = 0..n-1).  One block of NX * N threads;
@@ -54,8 +58,12 @@ __global__ void __launch_bounds__(256) powers_kernel(const float* K, int H, floa
 
 // One tick in the factorised form.  Dynamic shared memory: [track grid (race
 // car)] [V: H x ro_n float4, (a, b_1, b_2, b_3) coefficients per read-out].
+// Bound: issue (57 % of the slots; about 190 instructions per 32 steps of a candidate,
+// the track test most of them), with a quarter of the warps' time at the barriers of
+// the prologue and the reduction.  GB300, race car, N = 30001, H = 100: 30.0 us, 56.7
+// with 760 blocks of 128 threads that tested every listed segment of every step.
 template <int KIND>
-__global__ void __launch_bounds__(256) factored_kernel(const __grid_constant__ TickArgs a) {
+__global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_constant__ TickArgs a) {
   using B = BasisTraits<KIND>;
   constexpr int N = B::N, NX = B::NX, NU = B::NU, NP = B::NP;
   constexpr int ANG = (KIND == kBot) ? 0 : ((KIND == kCar) ? 2 : -1);
@@ -66,6 +74,14 @@ __global__ void __launch_bounds__(256) factored_kernel(const __grid_constant__ T
   if (fallback_not_needed(a)) return;
   const int n_eval = a.n_list ? *a.n_list : a.n_slots;
   const int H = a.horizon, ro_n = a.ro_n;
+  // every warp takes an equal share of the candidates, at most 32 at a time; the
+  // blocks that a short device-side list leaves without a share return at once
+  const int wpb = blockDim.x >> 5;
+  const int warps = (int)gridDim.x * wpb;
+  const int tile = max(1, min(32, (n_eval + warps - 1) / warps));
+  const int n_wtiles = (n_eval + tile - 1) / tile;
+  const int n_active = max(1, min((int)gridDim.x, (n_wtiles + wpb - 1) / wpb));
+  if ((int)blockIdx.x >= n_active) return;
 
   // the track grid arrives by bulk copy while the table V is built
   __shared__ uint64_t s_bar;
@@ -111,13 +127,26 @@ __global__ void __launch_bounds__(256) factored_kernel(const __grid_constant__ T
     const int t = e / ro_n, r = e - t * ro_n;
     const float* prow = a.ck + ((size_t)t * NX + a.ro_idx[r]) * N;
     float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;
-#pragma unroll 8
-    for (int j = 0; j < N; ++j) {
-      const float pj = __ldg(prow + j);
+    const auto add = [&](int j, float pj) {
       v0 = __fmaf_rn(pj, s_f[j][0], v0);
       v1 = __fmaf_rn(pj, s_f[j][1], v1);
       v2 = __fmaf_rn(pj, s_f[j][2], v2);
       v3 = __fmaf_rn(pj, s_f[j][3], v3);
+    };
+    if constexpr (N % 4 == 0) {  // rows of whole float4s: all of a row's loads in flight
+      float4 p4[N / 4];
+#pragma unroll
+      for (int j = 0; j < N / 4; ++j) p4[j] = __ldg(reinterpret_cast<const float4*>(prow) + j);
+#pragma unroll
+      for (int j = 0; j < N / 4; ++j) {
+        add(4 * j, p4[j].x);
+        add(4 * j + 1, p4[j].y);
+        add(4 * j + 2, p4[j].z);
+        add(4 * j + 3, p4[j].w);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < N; ++j) add(j, __ldg(prow + j));
     }
     V[e] = make_float4(v0, v1, v2, v3);
   }
@@ -141,16 +170,16 @@ __global__ void __launch_bounds__(256) factored_kernel(const __grid_constant__ T
 
   unsigned long long best = ~0ull;
   unsigned int n_safe = 0, n_exec = 0;
-  const int wpb = blockDim.x >> 5;
   // Time-parallel: the read-outs of different steps do not depend on each other,
-  // so a warp takes kFactCands candidates one after the other and tests 32 steps
-  // of a candidate at once (lane l: step t0 + l + 1); a ballot gives the first
-  // violation.
-  const int n_wtiles = failed ? 0 : (n_eval + kFactCands - 1) / kFactCands;
-  for (int wt = blockIdx.x * wpb + warp; wt < n_wtiles; wt += gridDim.x * wpb) {
-    // lanes 0..kFactCands-1 draw and score one candidate each
-    const int pos = wt * kFactCands + lane;
-    const bool valid = lane < kFactCands && pos < n_eval;
+  // so a warp takes its candidates one after the other and tests 32 steps of a
+  // candidate at once (lane l: step t0 + l + 1).  Only the first violation counts, so
+  // open positions (settle_open) are settled in the order of their steps, and none
+  // after a step that is known to violate.
+  for (int wt = failed ? n_wtiles : (int)blockIdx.x * wpb + warp; wt < n_wtiles; wt += warps) {
+    // lanes 0 .. tile - 1 draw and score one candidate each
+    const int pos = wt * tile + lane;
+    const int count = min(tile, n_eval - wt * tile);
+    const bool valid = lane < count;
     const int slot = (valid && a.slot_list) ? a.slot_list[pos] : pos;
     float xi[NU];
     if (valid) {
@@ -168,8 +197,7 @@ __global__ void __launch_bounds__(256) factored_kernel(const __grid_constant__ T
     float p[NP];
     monomials32<KIND>(xi, p);
     int my_ttv = 0;
-    for (int c = 0; c < kFactCands; ++c) {
-      if (!__shfl_sync(kFull, (int)valid, c)) continue;  // uniform over the warp
+    for (int c = 0; c < count; ++c) {
       float pc[NP];
 #pragma unroll
       for (int k = 0; k < NP; ++k) pc[k] = __shfl_sync(kFull, p[k], c);
@@ -177,9 +205,9 @@ __global__ void __launch_bounds__(256) factored_kernel(const __grid_constant__ T
       for (int t0 = 0; t0 < H; t0 += 32) {
         const int t = t0 + lane + 1;
         bool ok = true;
+        float px = 0.f, py = 0.f;
         if (t <= H) {
           const float4* Vt = V + (t - 1) * ro_n;
-          float px = 0.f, py = 0.f;
 #pragma unroll
           for (int r = 0; r < NX; ++r) {
             if (r < ro_n) {
@@ -192,12 +220,26 @@ __global__ void __launch_bounds__(256) factored_kernel(const __grid_constant__ T
               if (r == 1) py = v;
             }
           }
-          if constexpr (B::TRACK) {
-            if (track) ok = ok && track_ok<1>(a.safety.track, tv, px, py, 0, ok);
-          }
         }
-        const unsigned bad = __ballot_sync(kFull, !ok);
-        if (bad) {
+        unsigned int bad;
+        if (B::TRACK && track) {
+          const TrackCell cell = track_cell(a.safety.track, tv, px, py, ok && t <= H);
+          ok = ok && (cell.ok || cell.open || t > H);
+          bad = __ballot_sync(kFull, !ok);
+          unsigned int todo = __ballot_sync(kFull, cell.open), taken;
+          if (bad != 0u) todo &= (bad & (0u - bad)) - 1u;  // before the first violation
+          while (todo != 0u) {
+            const unsigned int got =
+                settle_open(a.safety.track, tv, px, py, cell, todo, &taken);
+            if ((taken & ~got) != 0u) {  // an earlier violation than any left open
+              bad |= taken & ~got;
+              break;
+            }
+          }
+        } else {
+          bad = __ballot_sync(kFull, !ok);
+        }
+        if (bad != 0u) {
           ttv = t0 + __ffs(bad) - 1;
           break;
         }
@@ -215,7 +257,8 @@ __global__ void __launch_bounds__(256) factored_kernel(const __grid_constant__ T
       if (a.cost_out) a.cost_out[slot] = cost;
     }
   }
-  session_epilogue<NU>(a, best, n_safe, n_exec, uh, failed);
+  session_epilogue<NU, TickArgs, kFactBlock / 32>(a, best, n_safe, n_exec, uh, failed,
+                                                  (unsigned int)n_active);
 }
 
 template <int KIND>
@@ -253,6 +296,10 @@ int launch_factored(mpmi_session* s, TickArgs& a, cudaStream_t st, int n_hint) {
   if (!fn) return fail(MPMI_E_UNSUPPORTED, "factored kernel not compiled for this basis");
   const size_t track = a.safety.has_track ? (size_t)a.safety.track.blob_bytes : 0;
   const size_t smem = track + (size_t)a.horizon * a.ro_n * sizeof(float4);
+  const int n_work = (n_hint > 0 && n_hint < s->n_slots) ? n_hint : s->n_slots;
+  // one candidate per warp until every SM has 32 warps: blocks of 4 to 32 warps
+  const int sms = s->ctx->sm_count;
+  const int wpb = std::max(4, std::min(kFactBlock / 32, (n_work + sms - 1) / sms));
   if (s->fact_grid == 0 || s->fact_smem != smem) {
     if (smem > 0) {
       const size_t cap = kMaxTrackBytes + (size_t)MPMI_MAX_HORIZON * MPMI_MAX_NX * sizeof(float4);
@@ -261,19 +308,17 @@ int launch_factored(mpmi_session* s, TickArgs& a, cudaStream_t st, int n_hint) {
       if (e != cudaSuccess) return fail(MPMI_E_CUDA, "cudaFuncSetAttribute (factored)");
     }
     int nb = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kFactBlock, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, 32 * wpb, smem);
     if (e != cudaSuccess || nb < 1)
       return fail(MPMI_E_UNSUPPORTED, "factored kernel cannot be resident");
-    s->fact_grid = nb * s->ctx->sm_count;
+    s->fact_grid = sms;
     s->fact_smem = smem;
   }
-  const int n_work = (n_hint > 0 && n_hint < s->n_slots) ? n_hint : s->n_slots;
-  const int n_wtiles = (n_work + kFactCands - 1) / kFactCands;
-  int grid = (n_wtiles + kFactBlock / 32 - 1) / (kFactBlock / 32);
+  int grid = (n_work + wpb - 1) / wpb;
   if (grid > s->fact_grid) grid = s->fact_grid;
   if (grid < 1) grid = 1;
   void* args[] = {&a};
-  const cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3(kFactBlock), args, smem, st);
+  const cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3(32 * wpb), args, smem, st);
   if (e != cudaSuccess)
     return fail(MPMI_E_CUDA, std::string("factored kernel launch: ") + cudaGetErrorString(e));
   return MPMI_OK;

@@ -425,67 +425,84 @@ __device__ __forceinline__ bool seg_hit(const DevTrack& tr, const TrackView& v, 
   return ex * ex + ey * ey < tr.w2;
 }
 
-// isSafe on the track part with one position per lane.  All 32 lanes of a warp call
-// it together (it votes and shuffles over the full warp; `active` says which lanes
-// have a position): never under a branch that some lanes skip.  A lane in a boundary cell tests the first two listed segments (nearest to the cell
-// first), which settles most positions on the road.  The warp then settles the
-// others together, four at a time: eight lanes test eight listed segments of one
-// position per round.  A lane that tests its whole list alone (7 to 15 entries when
-// the position is off the road) keeps the other 31 waiting through every round.
-// Race car, one lane per candidate: N = 16384 69 -> 64 us, N = 32768 95 -> 91 us, the
-// tensor-core rollout at N = 65536 79.7 -> 78.4 us.
-__device__ __forceinline__ bool track_ok_warp(const DevTrack& tr, const TrackView& v, float px,
-                                              float py, bool active) {
-  constexpr int FIRST = 2;
-  const int lane = threadIdx.x & 31;
-  bool ok = false, open = false;
-  int off = 0, cnt = 0;
+// isSafe on the track part with one position per lane, in two stages.  A lane in a
+// boundary cell tests the first two listed segments (nearest to the cell first), which
+// settles most positions on the road (track_cell).  The warp then settles the open
+// ones together, four at a time: eight lanes test eight listed segments of one
+// position per round (settle_open).  A lane that tests its whole list alone (7 to 15
+// entries when the position is off the road) keeps the other 31 waiting through every
+// round.  Race car, one lane per candidate: N = 16384 69 -> 64 us, N = 32768 95 -> 91
+// us, the tensor-core rollout at N = 65536 79.7 -> 78.4 us.
+struct TrackCell {
+  bool ok, open;  // on the road; undecided after the first two segments
+  int off, cnt;   // the cell's list
+};
+
+__device__ __forceinline__ TrackCell track_cell(const DevTrack& tr, const TrackView& v, float px,
+                                                float py, bool active) {
+  TrackCell r{false, false, 0, 0};
   if (active) {
     const float fx = (px - tr.gx0) * tr.inv_h;
     const float fy = (py - tr.gy0) * tr.inv_h;
     if ((fx >= 0.f) & (fx < (float)tr.gnx) & (fy >= 0.f) & (fy < (float)tr.gny)) {
       const uint32_t c = v.cells[(int)fy * tr.gnx + (int)fx];
       const uint32_t cls = c & 3u;
-      ok = cls == kCellInside;
+      r.ok = cls == kCellInside;
       if (cls == kCellBoundary) {
-        off = (int)((c >> 2) & 0x3FFFFFu);
-        cnt = (int)(c >> 24);
+        r.off = (int)((c >> 2) & 0x3FFFFFu);
+        r.cnt = (int)(c >> 24);
         // entries past the list's end repeat its last one (a list is never empty)
-        const bool h0 = seg_hit(tr, v, v.list[off], px, py);
-        const bool h1 = seg_hit(tr, v, v.list[off + min(1, cnt - 1)], px, py);
-        ok = h0 | h1;
-        open = !ok & (cnt > FIRST);
+        const bool h0 = seg_hit(tr, v, v.list[r.off], px, py);
+        const bool h1 = seg_hit(tr, v, v.list[r.off + min(1, r.cnt - 1)], px, py);
+        r.ok = h0 | h1;
+        r.open = !r.ok & (r.cnt > 2);
       }
     }
   }
-  unsigned int todo = __ballot_sync(kFull, open);
-  while (todo != 0u) {
-    // the next four open lanes, one per group of eight lanes (a group past the last
-    // one repeats it)
-    int src = __ffs(todo) - 1, mine = src;
-    todo &= todo - 1u;
+  return r;
+}
+
+// Takes up to four lanes off `todo` (not 0; lowest first), tests their positions and
+// returns the lanes on the road; *taken: the lanes tested.  All 32 lanes of a warp
+// call it together (it shuffles over the full warp): never under a branch that some
+// lanes skip.
+__device__ __forceinline__ unsigned int settle_open(const DevTrack& tr, const TrackView& v,
+                                                    float px, float py, const TrackCell& cell,
+                                                    unsigned int& todo, unsigned int* taken) {
+  const int lane = threadIdx.x & 31;
+  // one open lane per group of eight lanes (a group past the last one repeats it)
+  const unsigned int before = todo;
+  int src = __ffs(todo) - 1, mine = src;
+  todo &= todo - 1u;
 #pragma unroll
-    for (int k = 1; k < 4; ++k) {
-      if (todo != 0u) {
-        src = __ffs(todo) - 1;
-        todo &= todo - 1u;
-      }
-      if ((lane >> 3) >= k) mine = src;
+  for (int k = 1; k < 4; ++k) {
+    if (todo != 0u) {
+      src = __ffs(todo) - 1;
+      todo &= todo - 1u;
     }
-    const float qx = __shfl_sync(kFull, px, mine), qy = __shfl_sync(kFull, py, mine);
-    const int qo = __shfl_sync(kFull, off, mine), qc = __shfl_sync(kFull, cnt, mine);
-    bool hit = false;
-    for (int i = FIRST + (lane & 7); i < qc && !hit; i += 16) {
-      const bool h0 = seg_hit(tr, v, v.list[qo + i], qx, qy);
-      const bool h1 = seg_hit(tr, v, v.list[qo + min(i + 8, qc - 1)], qx, qy);
-      hit = h0 | h1;
-    }
-    __syncwarp();
-    // every lane with a hit names the position it tested
-    const unsigned int got = __reduce_or_sync(kFull, hit ? 1u << mine : 0u);
-    ok = ok | (((got >> lane) & 1u) != 0u);
+    if ((lane >> 3) >= k) mine = src;
   }
-  return ok;
+  *taken = before & ~todo;
+  const float qx = __shfl_sync(kFull, px, mine), qy = __shfl_sync(kFull, py, mine);
+  const int qo = __shfl_sync(kFull, cell.off, mine), qc = __shfl_sync(kFull, cell.cnt, mine);
+  bool hit = false;
+  for (int i = 2 + (lane & 7); i < qc && !hit; i += 16) {
+    const bool h0 = seg_hit(tr, v, v.list[qo + i], qx, qy);
+    const bool h1 = seg_hit(tr, v, v.list[qo + min(i + 8, qc - 1)], qx, qy);
+    hit = h0 | h1;
+  }
+  // every lane with a hit names the position it tested
+  return __reduce_or_sync(kFull, hit ? 1u << mine : 0u);
+}
+
+// Both stages; all 32 lanes of a warp call it together, `active` says which have a
+// position.
+__device__ __forceinline__ bool track_ok_warp(const DevTrack& tr, const TrackView& v, float px,
+                                              float py, bool active) {
+  TrackCell cell = track_cell(tr, v, px, py, active);
+  unsigned int todo = __ballot_sync(kFull, cell.open), got = 0u, taken;
+  while (todo != 0u) got |= settle_open(tr, v, px, py, cell, todo, &taken);
+  return cell.ok | (((got >> (threadIdx.x & 31)) & 1u) != 0u);
 }
 
 // isSafe on the track part, shared by the L lanes of a group: lane q tests list
