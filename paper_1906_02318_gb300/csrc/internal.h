@@ -155,6 +155,7 @@ struct mpmi_session {
   const mpmi_model* model = nullptr;
   mpmi_session_config cfg{};
   int n_slots = 0, lanes = 1, cands = 1, block = 128, grid_g = 0;
+  bool auto_lanes = false;  // lanes and candidates per thread were left to the library
   // resident blocks on the device per launch kind (plain or trajectories, all
   // slots or the few-candidate shape, with or without noise) and the dynamic
   // shared memory they assume

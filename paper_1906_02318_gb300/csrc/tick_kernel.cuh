@@ -352,14 +352,11 @@ __device__ __forceinline__ void candidate_value(const P& a, int slot, const floa
 // Two standard normals from two Philox words (Box & Muller, Ann. Math. Stat. 29,
 // 1958): u1 = ((w_a >> 8) + 1) 2^-24 in (0, 1], u2 = (w_b >> 8) 2^-24 in [0, 1),
 // both exact in binary32; n = sqrt(-2 ln u1) (cos 2 pi u2, sin 2 pi u2).
-__device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, float& n0, float& n1) {
-  const float u1 = (float)((wa >> 8) + 1u) * 0x1p-24f;
-  const float u2 = (float)(wb >> 8) * 0x1p-24f;
-  const float r = sqrtf(-2.f * logf(u1));
-  float s, c;
-  sincospif(2.f * u2, &s, &c);
-  n0 = r * c;
-  n1 = r * s;
+__device__ __forceinline__ float box_muller_sq(uint32_t wa) {  // -2 ln u1
+  return -2.f * logf((float)((wa >> 8) + 1u) * 0x1p-24f);
+}
+__device__ __forceinline__ void box_muller_angle(uint32_t wb, float& s, float& c) {
+  sincospif(2.f * ((float)(wb >> 8) * 0x1p-24f), &s, &c);
 }
 
 // Alg. 2's noise z_i after prediction step t of candidate `slot`: the state
@@ -367,22 +364,60 @@ __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, float& n0, 
 // one Philox call with counter (slot, tick lo, (tick hi mod 2^16) + 2^16 t +
 // 2^25 b, stream); its words pair as (w0, w1) -> 4b, 4b+1 and (w2, w3) -> 4b+2,
 // 4b+3.  Since t >= 1 these counters never meet a candidate counter.
-template <int NX, class P>
-__device__ __forceinline__ void add_noise(const P& a, TickDyn d, int slot, int t, float* z) {
+// noise_normals gives the n_j (of the blocks in use), apply_noise adds them to z.
+// Steps t, t + by, ... (S of them) at once, every stage for all of them before the
+// next: the square root's rare-case branch would otherwise keep their chains apart.
+template <int NX, int S, class P>
+__device__ __forceinline__ void noise_normals(const P& a, TickDyn d, int slot, int t, int by,
+                                              float (*n)[NX]) {
   constexpr int NB = (NX + 3) / 4;
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
     if (4 * b < a.n_noise) {
-      const uint32_t c2 = (d.t_hi & 0xFFFFu) + ((uint32_t)t << 16) + ((uint32_t)b << 25);
-      const U32x4 w = philox4x32_10(U32x4{(uint32_t)slot, d.t_lo, c2, a.stream}, a.key0, a.key1);
-      float n[4];
-      box_muller(w.x, w.y, n[0], n[1]);
-      box_muller(w.z, w.w, n[2], n[3]);
+      U32x4 w[S];
+      float r[S][2], sn[S][2], cs[S][2];
 #pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (4 * b + j < NX) z[4 * b + j] = __fmaf_rn(a.noise_sigma[4 * b + j], n[j], z[4 * b + j]);
+      for (int s = 0; s < S; ++s) {
+        const uint32_t c2 = (d.t_hi & 0xFFFFu) + ((uint32_t)(t + s * by) << 16) + ((uint32_t)b << 25);
+        w[s] = philox4x32_10(U32x4{(uint32_t)slot, d.t_lo, c2, a.stream}, a.key0, a.key1);
+      }
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        r[s][0] = box_muller_sq(w[s].x);
+        r[s][1] = box_muller_sq(w[s].z);
+      }
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        box_muller_angle(w[s].y, sn[s][0], cs[s][0]);
+        box_muller_angle(w[s].w, sn[s][1], cs[s][1]);
+      }
+#pragma unroll
+      for (int s = 0; s < S; ++s) {
+        r[s][0] = sqrtf(r[s][0]);
+        r[s][1] = sqrtf(r[s][1]);
+      }
+#pragma unroll
+      for (int s = 0; s < S; ++s)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (4 * b + j < NX)
+            n[s][4 * b + j] = r[s][j >> 1] * ((j & 1) ? sn[s][j >> 1] : cs[s][j >> 1]);
     }
   }
+}
+
+template <int NX, class P>
+__device__ __forceinline__ void apply_noise(const P& a, const float* n, float* z) {
+#pragma unroll
+  for (int j = 0; j < NX; ++j)
+    if ((j & ~3) < a.n_noise) z[j] = __fmaf_rn(a.noise_sigma[j], n[j], z[j]);
+}
+
+template <int NX, class P>
+__device__ __forceinline__ void add_noise(const P& a, TickDyn d, int slot, int t, float* z) {
+  float n[1][NX];
+  noise_normals<NX, 1>(a, d, slot, t, 1, n);
+  apply_noise<NX>(a, n[0], z);
 }
 
 // Input monomials p_k(xi) of the split lifting, float32.
@@ -755,6 +790,16 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
 #pragma unroll
       for (int j = 0; j < KP::NF / 2; ++j) kreg[pp][j] = sK4[pair_of(pp) * KP::STRIDE + j];
   }
+  // The noise does not depend on z, and one step's Philox rounds and Box-Muller
+  // functions are a longer chain than the step itself, so AHEAD steps' normals are
+  // drawn at once: a group of L lanes draws L steps, one per lane (every lane drew
+  // every step's before), and one lane with K in registers draws four, their chains
+  // side by side (the race car's one-lane shapes have no registers left for that).
+  // Normals past the horizon are drawn and not used.  GB300: balance bot H = 50,
+  // N = 1000 (4 lanes) 27.3 -> 15 us, N = 16384 (1 lane) 27.1 -> 22.9; race car H = 60,
+  // N = 1024 (16 lanes) 60 -> 30 us, N = 4096 (8) 76 -> 44, N = 16384 (2) 97 -> 80.
+  constexpr int AHEAD = !NOISE ? 1 : (L > 1 ? L : (KIND != kCar && C == 1 ? 4 : 1));
+  float ahead[AHEAD >= L ? AHEAD / L : 1][NX];
   for (int t = 1; t <= H; ++t) {
     if constexpr (PK) {
       // z <- K z with the free rows in pairs (see KPair): per pair one chain of
@@ -946,7 +991,27 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
         z[0][k] = v.x; z[0][k + 1] = v.y; z[0][k + 2] = v.z; z[0][k + 3] = v.w;
       }
     }
-    if constexpr (NOISE) {
+    if constexpr (NOISE && AHEAD > 1) {
+      // lane q of the group draws steps t + q, t + L + q, ..., and each step reads its
+      // lane's normals
+      const int at = (t - 1) & (AHEAD - 1);
+      if (at == 0) noise_normals<NX, AHEAD / L>(a, d, slot[0], t + q, L, ahead);
+      if constexpr (L > 1) {
+        float n[NX];
+#pragma unroll
+        for (int j = 0; j < NX; ++j)
+          n[j] = __shfl_sync(kFull, ahead[0][j], (lane & ~(L - 1)) + (at & (L - 1)));
+        apply_noise<NX>(a, n, z[0]);
+      } else {
+        apply_noise<NX>(a, ahead[0], z[0]);
+      }
+      if (AHEAD > L && (at & (L - 1)) == L - 1) {
+#pragma unroll
+        for (int s = 0; s + 1 < AHEAD / L; ++s)
+#pragma unroll
+          for (int j = 0; j < NX; ++j) ahead[s][j] = ahead[s + 1][j];
+      }
+    } else if constexpr (NOISE) {
 #pragma unroll
       for (int c = 0; c < C; ++c)
         if (alive[c]) add_noise<NX>(a, d, slot[c], t, z[c]);
