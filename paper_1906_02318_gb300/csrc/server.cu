@@ -2,12 +2,13 @@
 // its own N, H, sampler stream and tick counter, evaluated together in one
 // persistent launch that is replayed from a CUDA graph.
 //
-// Device side: the batch table lists the requests; their warp-tiles form one index
-// space (prefix sums in tile_begin).  Persistent warps stride over it; each
-// warp-tile runs the same per-tile code as the single-session tick (run_tile),
-// then folds its key and counts into the session's reduction record; the warp
-// that completes a session's last tile decodes its result.  A session's outcome
-// is therefore bit-identical whether it is served alone or in a mix.
+// Device side: the batch table lists the requests.  In a small batch their warp-tiles
+// form one index space that persistent warps stride over; in a large one their sorted
+// units do, and the blocks take units from a counter.  Either way a tile runs the same
+// code as the single-session tick (run_tile), its key and counts are folded into the
+// session's reduction record, and whoever completes a session's last tile or unit
+// decodes its result.  A session's outcome is therefore bit-identical whether it is
+// served alone or in a mix.
 //
 // Host side: admission (a free session slot and room in the context's memory
 // budget), kBuffers batch buffers, each with one captured graph (table upload,
@@ -37,7 +38,10 @@ struct SessionTick {
   double in_lo64[MPMI_MAX_NU], in_hi64[MPMI_MAX_NU];
   uint32_t key0, key1, t_lo, t_hi, stream, pad0;
   const float* ext;
-  int horizon, n_tiles, tile_begin, pad1;
+  int horizon, n_takes;
+  // range i of the batch, in the order it is served (entry i holds range i, which is
+  // another request's in general): its first tile or unit and its request
+  int range_begin, range_entry;
   const int* slot_list;
   const int* n_list;
   int32_t* ttv_out;
@@ -53,8 +57,9 @@ struct SessionTick {
 
 struct ServeHeader {
   int n_requests;
-  int total_tiles;
-  int pad[2];
+  int total;  // tiles or units
+  int unit;   // slots per sorted unit, 0: the warps stride over unsorted tiles
+  int next;   // next unit to take (device; the upload resets it)
 };
 
 struct ServeArgs {
@@ -62,8 +67,31 @@ struct ServeArgs {
   const float* Ks;  // K with each row's columns in staging order
   const float* Kp;  // the free rows of K in pairs (KPair layout; race car)
   DevSafety safety;
-  const ServeHeader* table;  // header followed by SessionTick entries
+  ServeHeader* table;  // header followed by SessionTick entries
 };
+
+constexpr int kServeUnit = 4096;  // most slots of a unit
+
+// Folds one tile's or unit's minimum and counts into its session's reduction record;
+// whoever completes the session's last one decodes the result and resets the record.
+template <int NU>
+__device__ __forceinline__ void fold_take(const SessionTick& st, unsigned long long best,
+                                          unsigned long long cnt, const float* uh) {
+  TickScratch* sc = st.scratch;
+  atomicMin(&sc->key, best);
+  atomicAdd(&sc->counts, cnt);
+  // acquire-release on the counter orders these atomics before the increment and lets
+  // the last one see every other's
+  unsigned int prev;
+  asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(prev) : "l"(&sc->done) : "memory");
+  if (prev != (unsigned int)st.n_takes - 1) return;
+  const unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&sc->key);
+  const unsigned long long c = *reinterpret_cast<volatile unsigned long long*>(&sc->counts);
+  write_result<NU>(st, k, c, uh);
+  sc->key = ~0ull;
+  sc->counts = 0ull;
+  sc->done = 0u;
+}
 
 template <int KIND, int L, int C, bool KSMEM>
 __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_constant__ ServeArgs sa) {
@@ -79,10 +107,12 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
   __shared__ __align__(16) float s_x[(L > 1) ? NW : 1][2][GPW][S];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int q = lane % L;
-  // the grid covers the largest batch; a block past the batch's warp-tiles leaves
-  // before staging anything, so that a small batch holds few SMs and batches in
-  // flight at the same time share the device
-  if ((long long)blockIdx.x * (blockDim.x >> 5) >= (long long)sa.table->total_tiles) return;
+  // the grid covers the largest batch; a block past the batch's work leaves before
+  // staging anything, so that a small batch holds few SMs and batches in flight at the
+  // same time share the device
+  ServeHeader* hdr = sa.table;
+  const int total = hdr->total, unit = hdr->unit, n_req = hdr->n_requests;
+  if ((long long)blockIdx.x * (unit ? 1 : blockDim.x >> 5) >= (long long)total) return;
 
   if constexpr (PK) {
     const uint4* src = reinterpret_cast<const uint4*>(sa.Kp);
@@ -115,61 +145,100 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
   }
   if constexpr (KSMEM || B::TRACK) __syncthreads();
 
-  const ServeHeader* hdr = sa.table;
-  const int n_req = hdr->n_requests, total = hdr->total_tiles;
   const SessionTick* ent = reinterpret_cast<const SessionTick*>(hdr + 1);
-  const int wpb = blockDim.x >> 5;
+  constexpr int PER_WARP = GPW * C;
   int cur = -1;
   float xs[NX], uh[NU], sn = 0.f, cs = 1.f;
-  for (int gwt = blockIdx.x * wpb + warp; gwt < total; gwt += gridDim.x * wpb) {
-    // the request this warp-tile belongs to (warp-uniform binary search)
+  // the range that tile or unit u belongs to (binary search over the ranges' starts)
+  const auto range_of = [&](int u) {
     int lo = 0, hi = n_req - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
-      if (ent[mid].tile_begin <= gwt) lo = mid;
+      if (ent[mid].range_begin <= u) lo = mid;
       else hi = mid - 1;
     }
-    const SessionTick& st = ent[lo];
-    if (lo != cur) {
+    return lo;
+  };
+  const auto load_state = [&](const SessionTick& st, int req) {
+    if (req == cur) return;
 #pragma unroll
-      for (int j = 0; j < NX; ++j) xs[j] = __double2float_rn(st.x_t_buf[j]);
+    for (int j = 0; j < NX; ++j) xs[j] = __double2float_rn(st.x_t_buf[j]);
 #pragma unroll
-      for (int j = 0; j < NU; ++j) uh[j] = __double2float_rn(st.u_h_buf[j]);
-      if constexpr (ANG >= 0) sincosf(xs[ANG], &sn, &cs);
-      cur = lo;
-    }
-    unsigned long long best = ~0ull;
-    unsigned int n_safe = 0, n_exec = 0;
-    run_tile<KIND, L, C, KSMEM, false, false, true>(st, dyn_of(st), sa.safety, gwt - st.tile_begin, st.n_slots, xs, uh,
-                                       sn, cs, kr, sK4, tv, &s_x[L > 1 ? warp : 0][0][0][0],
-                                       best, n_safe, n_exec);
+    for (int j = 0; j < NU; ++j) uh[j] = __double2float_rn(st.u_h_buf[j]);
+    if constexpr (ANG >= 0) sincosf(xs[ANG], &sn, &cs);
+    cur = req;
+  };
+  if (unit == 0) {
+    const int wpb = blockDim.x >> 5;
+    for (int gwt = blockIdx.x * wpb + warp; gwt < total; gwt += gridDim.x * wpb) {
+      const int r = range_of(gwt), req = ent[r].range_entry;
+      const SessionTick& st = ent[req];
+      load_state(st, req);
+      unsigned long long best = ~0ull;
+      unsigned int n_safe = 0, n_exec = 0;
+      run_tile<KIND, L, C, KSMEM, false, false, true>(
+          st, dyn_of(st), sa.safety, gwt - ent[r].range_begin, st.n_slots, xs, uh, sn, cs, kr, sK4,
+          tv, &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long other = __shfl_xor_sync(kFull, best, o);
-      best = other < best ? other : best;
-      n_exec += __shfl_xor_sync(kFull, n_exec, o);
-      n_safe += __shfl_xor_sync(kFull, n_safe, o);
-    }
-    if (lane == 0) {
-      TickScratch* sc = st.scratch;
-      atomicMin(&sc->key, best);
-      atomicAdd(&sc->counts, ((unsigned long long)n_safe << 40) + n_exec);
-      // acquire-release on the tile counter orders this warp's atomics before the
-      // increment and lets the last warp see every other warp's
-      unsigned int prev;
-      asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(prev) : "l"(&sc->done) : "memory");
-      if (prev == (unsigned int)st.n_tiles - 1) {
-        // this warp finished the session's last tile: decode and reset its record
-        const unsigned long long k = *reinterpret_cast<volatile unsigned long long*>(&sc->key);
-        const unsigned long long cnt =
-            *reinterpret_cast<volatile unsigned long long*>(&sc->counts);
-        write_result<NU>(st, k, cnt, uh);
-        sc->key = ~0ull;
-        sc->counts = 0ull;
-        sc->done = 0u;
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(kFull, best, o);
+        best = other < best ? other : best;
+        n_exec += __shfl_xor_sync(kFull, n_exec, o);
+        n_safe += __shfl_xor_sync(kFull, n_safe, o);
       }
+      if (lane == 0) fold_take<NU>(st, best, ((unsigned long long)n_safe << 40) + n_exec, uh);
+      __syncwarp();
     }
-    __syncwarp();
+    return;
+  }
+  if constexpr (L == 1) {
+    char* buf = reinterpret_cast<char*>(s_dyn + KWORDS) +
+                (B::TRACK && sa.safety.has_track ? sa.safety.track.blob_bytes : 0);
+    __shared__ int s_unit, s_tile;
+    __shared__ unsigned long long s_best, s_cnt;
+    if (tid == 0) s_unit = atomicAdd(&hdr->next, 1);
+    while (true) {
+      __syncthreads();  // s_unit is set; the previous unit's results are taken
+      const int u = s_unit;
+      if (u >= total) break;
+      const int r = range_of(u), req = ent[r].range_entry;
+      const SessionTick& st = ent[req];
+      const int base = (u - ent[r].range_begin) * unit;
+      const int cnt = min(unit, st.n_slots - base);
+      load_state(st, req);
+      const uint16_t* order = sort_unit<NU>(st, dyn_of(st), base, cnt, unit, uh, buf, &s_tile);
+      __syncthreads();
+      if (tid == 0) {
+        s_unit = atomicAdd(&hdr->next, 1);  // read after the unit's last barrier
+        s_best = ~0ull;
+        s_cnt = 0ull;
+      }
+      __syncthreads();
+      unsigned long long best = ~0ull;
+      unsigned int n_safe = 0, n_exec = 0;
+      while (true) {
+        int wt = 0;
+        if (lane == 0) wt = atomicAdd(&s_tile, 1);
+        wt = __shfl_sync(kFull, wt, 0);
+        if (wt * PER_WARP >= cnt) break;
+        run_tile<KIND, L, C, KSMEM, false, false, true>(
+            st, dyn_of(st), sa.safety, wt, cnt, xs, uh, sn, cs, kr, sK4, tv,
+            &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec, order, base);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long other = __shfl_xor_sync(kFull, best, o);
+        best = other < best ? other : best;
+        n_exec += __shfl_xor_sync(kFull, n_exec, o);
+        n_safe += __shfl_xor_sync(kFull, n_safe, o);
+      }
+      if (lane == 0) {
+        atomicMin(&s_best, best);
+        atomicAdd(&s_cnt, ((unsigned long long)n_safe << 40) + n_exec);
+      }
+      __syncthreads();
+      if (tid == 0) fold_take<NU>(st, s_best, s_cnt, uh);
+    }
   }
 }
 
@@ -214,6 +283,12 @@ static std::vector<ServeKernel> serve_shapes(int kind) {
     case kLin41: return {make_serve<kLin41, 1, 1, false>()};
   }
   return {};
+}
+
+// Dynamic shared memory of a shape: K, the track grid, and a sorted unit.
+static size_t serve_smem(const ServeKernel& k, const DevSafety& safety) {
+  return k.k_smem + (safety.has_track ? (size_t)safety.track.blob_bytes : 0) +
+         (k.lanes == 1 ? unit_bytes(kServeUnit) : 0);
 }
 
 static ServeKernel pick_serve(int kind) {
@@ -293,6 +368,48 @@ static int build_graph(mpmi_server* s, int b) {
   return MPMI_OK;
 }
 
+// Lays out the staged requests: as tiles that the warps stride over, or, where the
+// one-lane shapes have several tiles per warp, as sorted units (sort_unit) that the
+// blocks take from a counter, ordered by horizon, longest first, so that the units
+// taken last are short ones.  Below two tiles per warp the race car loses by a unit's
+// barriers (93k slots 245 -> 274 us), below four the balance bot does (107 us either
+// way).  Mixed sizes and horizons (N log-uniform in 1k..64k, H in 20..100), untuned
+// servers, submit to collect: 24 race cars 850 -> 702 us, 60 2320 -> 1860; 24 balance
+// bots 210 -> 168, 60 455 -> 336; both servers together, 48 sessions 1077 -> 806.  One
+// to six units per block measured the same within 2 % from two on.
+static void plan_batch(mpmi_server* s, ServeHeader* hdr) {
+  SessionTick* ent = reinterpret_cast<SessionTick*>(hdr + 1);
+  const int n = hdr->n_requests;
+  const ServeKernel& k = s->kern;
+  long long slots = 0;
+  for (int i = 0; i < n; ++i) slots += ent[i].n_slots;
+  std::vector<int> by(n);
+  for (int i = 0; i < n; ++i) by[i] = i;
+  const long long warps = (long long)s->grid * (s->block / 32);
+  const int min_tiles = s->model->kind == kCar ? 2 : 4;  // per warp
+  hdr->unit = 0;
+  if (k.lanes == 1 && slots >= min_tiles * warps * k.per_warp) {
+    std::stable_sort(by.begin(), by.end(),
+                     [&](int a, int b) { return ent[a].horizon > ent[b].horizon; });
+    // a multiple of one tile per warp of a block, about three units per block
+    const int step = k.per_warp * (s->block / 32);
+    const long long want = slots / (3LL * s->grid);
+    hdr->unit = (int)std::min<long long>(kServeUnit / step,
+                                         std::max<long long>(1, (want + step / 2) / step)) * step;
+  }
+  const int per = hdr->unit ? hdr->unit : k.per_warp;
+  int begin = 0;
+  for (int i = 0; i < n; ++i) {
+    SessionTick& e = ent[by[i]];
+    e.n_takes = (e.n_slots + per - 1) / per;
+    ent[i].range_begin = begin;
+    ent[i].range_entry = by[i];
+    begin += e.n_takes;
+  }
+  hdr->total = begin;
+  hdr->next = 0;
+}
+
 static int n_flying(const mpmi_server* s) {
   int n = 0;
   for (int b = 0; b < kServeBuffers; ++b) n += s->flying[b] ? 1 : 0;
@@ -338,7 +455,7 @@ int mpmi_server_create(mpmi_ctx* ctx, const mpmi_model* model, int32_t max_sessi
   s->used.assign(max_sessions, 0);
   s->state.assign(max_sessions, 0);
   s->table_bytes = sizeof(ServeHeader) + sizeof(SessionTick) * (size_t)max_sessions;
-  s->smem = kern.k_smem + (model->dev_safety.has_track ? (size_t)model->dev_safety.track.blob_bytes : 0);
+  s->smem = serve_smem(kern, model->dev_safety);
   s->per_session_bytes =
       sizeof(TickScratch) + kServeBuffers * (sizeof(SessionTick) + sizeof(mpmi_result));
   const uint64_t fixed =
@@ -490,8 +607,6 @@ int mpmi_server_submit(mpmi_server* s, int32_t n, const int32_t* slots, const do
     e.t_hi = (uint32_t)(ticks[r] >> 32);
     e.stream = c.stream_id;
     e.horizon = c.horizon;
-    e.n_tiles = (e.n_slots + s->kern.per_warp - 1) / s->kern.per_warp;
-    e.tile_begin = hdr->total_tiles;
     e.tick = ticks[r];
     e.scratch = s->scratch + sl;
     e.result = s->res_dev[s->stage] + i;
@@ -501,7 +616,6 @@ int mpmi_server_submit(mpmi_server* s, int32_t n, const int32_t* slots, const do
         dev_base + sizeof(ServeHeader) + sizeof(SessionTick) * (size_t)i +
         offsetof(SessionTick, u_h_buf));
     hdr->n_requests += 1;
-    hdr->total_tiles += e.n_tiles;
     s->slots[s->stage].push_back(sl);
     s->state[sl] = 1;
   }
@@ -517,6 +631,7 @@ int mpmi_server_launch(mpmi_server* s, void* stream, int32_t* n_launched) {
   if (n_flying(s) >= s->max_in_flight)
     return fail(MPMI_E_NOT_READY, "server_launch: the most batches allowed in flight are on the "
                                   "GPU (collect one first)");
+  plan_batch(s, s->table_host[b]);
   // the batch follows the work queued so far on the caller's stream, and runs
   // on its buffer's own stream so that it overlaps the batches in flight
   cudaStream_t st = (cudaStream_t)stream;
@@ -541,7 +656,7 @@ int mpmi_server_launch(mpmi_server* s, void* stream, int32_t* n_launched) {
   }
   s->stage = nb;
   s->table_host[nb]->n_requests = 0;
-  s->table_host[nb]->total_tiles = 0;
+  s->table_host[nb]->total = 0;
   s->slots[nb].clear();
   return MPMI_OK;
 }
@@ -605,7 +720,7 @@ int mpmi_server_collect(mpmi_server* s, mpmi_result* out, int32_t* slots_out, in
   for (int sl : s->slots[b]) s->state[sl] = 0;
   s->slots[b].clear();
   s->table_host[b]->n_requests = 0;
-  s->table_host[b]->total_tiles = 0;
+  s->table_host[b]->total = 0;
   s->flying[b] = false;
   return MPMI_OK;
 }
@@ -617,8 +732,7 @@ namespace mpmi {
 // Switches the server to launch shape k with `block` threads per block and
 // re-captures both batch graphs.  UNSUPPORTED if the shape cannot be resident.
 static int server_set_shape(mpmi_server* s, const ServeKernel& k, int block) {
-  const size_t smem =
-      k.k_smem + (s->model->dev_safety.has_track ? (size_t)s->model->dev_safety.track.blob_bytes : 0);
+  const size_t smem = serve_smem(k, s->model->dev_safety);
   if (smem > 0 &&
       cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
           cudaSuccess) {

@@ -78,3 +78,35 @@ def test_caller_samples_outside_the_box(setup, which):
         out.append(run_gpu(lib, s, x_t, u_h, candidates=cd))
         s.close()
     _same(*out)
+
+
+@pytest.mark.parametrize("which,sizes", [
+    ("car", [(60001, 30), (40000, 60), (0, 25), (5000, 100), (33333, 20)]),
+    ("bot", [(65536, 50), (65535, 20), (1, 60), (64, 50), (65000, 100), (50001, 35), (33, 90)])])
+def test_served_units_equal_the_tick_alone(setup, which, sizes):
+    """A batch large enough to be served as sorted units: every session's result is that
+    of its tick alone, over two batches (other states, other candidates)."""
+    import torch
+    lib, ctx, envs = setup
+    env, model = envs[which]
+    srv = lib.Server(ctx, model, 8)
+    slots = [srv.admit(n, h, env.lo, env.hi, seed=50 + i, stream_id=i)
+             for i, (n, h) in enumerate(sizes)]
+    rng = np.random.default_rng(4)
+    for batch in range(2):
+        x = (rng.uniform([-0.2, -0.6, -1, -0.8], [0.2, 0.6, 1, 0.8], (len(sizes), 4))
+             if which == "bot" else data.car_start_state(env.track, vx=12.0)
+             + rng.uniform(-1, 1, (len(sizes), 6)) * [2, 2, 0.1, 4, 0.3, 0.3])
+        u = data.to_f32_exact(rng.uniform(env.lo, env.hi, (len(sizes), len(env.lo))))
+        ticks = [1000 * batch + i for i in range(len(sizes))]
+        srv.submit(slots, x, u, ticks)
+        srv.launch()
+        got = dict(srv.collect())
+        for i, (n, h) in enumerate(sizes):
+            s = lib.Session(ctx, model, n, h, env.lo, env.hi, seed=50 + i, stream_id=i, lanes=2)
+            want = run_gpu(lib, s, x[i], u[i], tick=ticks[i])["result"]
+            s.close()
+            for k in ("index", "status", "n_safe", "ttv", "cost", "executed_steps", "n_slots"):
+                assert got[slots[i]][k] == want[k], (i, k)
+            assert np.array_equal(got[slots[i]]["u_r"], want["u_r"])
+    srv.free()
