@@ -54,11 +54,11 @@ static TickKernel pick_tick(int kind, int lanes, int cands, bool traj, bool nois
 // Default launch shape (lanes, candidates per thread, block).  A tick is one
 // warp's serial chain of H steps until the candidates fill the GPU several times
 // over, so few candidates take more lanes each.  Measured on GB300 (race car,
-// H = 60, CUDA events, L2 flushed): N = 1024 16 lanes 28 us; N = 4096 8 lanes
-// 38 us against 47 (2 lanes) and 69 (1 lane); N = 8192 2 lanes 47 us against 62
-// (8 lanes) and 69; N = 16384 2 lanes 60 us against 69 (1 lane); N = 32768 1 lane
-// 103 us against 110 (2 lanes); past eight tiles per SM (38,912 slots) two candidates
-// per thread (N = 40000 124 us against 131).  The
+// H = 60, ticks back to back): N = 1024 16 lanes 20.8 us, 8 lanes 22.8, 2 lanes 35;
+// N = 4096 8 lanes 31 against 39 (16) and 35 (2); N = 5000 2 lanes 35 against 45 (8);
+// N = 16384 2 lanes 53 against 60 (1 lane) and 88 (two candidates per thread); N =
+// 32768 1 lane 89 against 98 (2 lanes); past eight tiles per SM (38,912 slots) two
+// candidates per thread (N = 40000 124 us against 131).  The
 // two-lane shape keeps two warps per SM sub-partition while they fit one wave
 // (two 128-thread blocks per SM), hiding each other's latency.  Balance bot
 // N <= 4096 with 4 lanes 12.6 against 13.4..14.1 us, else one lane.  Blocks of

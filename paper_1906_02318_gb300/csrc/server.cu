@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
       load_state(st, req);
       unsigned long long best = ~0ull;
       unsigned int n_safe = 0, n_exec = 0;
-      run_tile<KIND, L, C, KSMEM, false, false, true>(
+      run_tile<KIND, L, C, KSMEM, false, false, true, false>(
           st, dyn_of(st), sa.safety, gwt - ent[r].range_begin, st.n_slots, xs, uh, sn, cs, kr, sK4,
           tv, &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec);
 #pragma unroll
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
         if (lane == 0) wt = atomicAdd(&s_tile, 1);
         wt = __shfl_sync(kFull, wt, 0);
         if (wt * PER_WARP >= cnt) break;
-        run_tile<KIND, L, C, KSMEM, false, false, true>(
+        run_tile<KIND, L, C, KSMEM, false, false, true, false>(
             st, dyn_of(st), sa.safety, wt, cnt, xs, uh, sn, cs, kr, sK4, tv,
             &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec, order, base);
       }

@@ -530,6 +530,65 @@ __device__ __forceinline__ unsigned int settle_open(const DevTrack& tr, const Tr
   return __reduce_or_sync(kFull, hit ? 1u << mine : 0u);
 }
 
+// The first stage without branches, for code that runs it beside other work; an
+// inactive lane reads entry 0 of the lists.  L = 2: the two lanes of a candidate test
+// one of the first two segments each; L >= 8: a candidate's lanes test the first
+// sixteen segments (track_settle joins them).
+template <int L>
+__device__ __forceinline__ TrackCell track_front(const DevTrack& tr, const TrackView& v, float px,
+                                                 float py, bool active, int q) {
+  const float fx = (px - tr.gx0) * tr.inv_h;
+  const float fy = (py - tr.gy0) * tr.inv_h;
+  const bool in = active & (fx >= 0.f) & (fx < (float)tr.gnx) & (fy >= 0.f) & (fy < (float)tr.gny);
+  const int ix = (int)fx, iy = (int)fy;
+  const uint32_t c = v.cells[in ? iy * tr.gnx + ix : 0];
+  const uint32_t cls = in ? c & 3u : (uint32_t)kCellOutside;
+  const bool edge = cls == kCellBoundary;
+  TrackCell r;
+  r.off = edge ? (int)((c >> 2) & 0x3FFFFFu) : 0;
+  r.cnt = edge ? (int)(c >> 24) : 1;
+  constexpr int FIRST = L <= 2 ? 2 : 16;  // segments the candidate's lanes test here
+  bool hit = false;
+#pragma unroll
+  for (int i = 0; i < FIRST / L; ++i)
+    hit = hit | seg_hit(tr, v, v.list[r.off + min(q + i * L, r.cnt - 1)], px, py);
+  r.ok = (cls == kCellInside) | (edge & hit);
+  r.open = edge & !hit & (r.cnt > FIRST);
+  return r;
+}
+
+// The second stage for track_front's answer, by whole warps.
+template <int L>
+__device__ __forceinline__ bool track_settle(const DevTrack& tr, const TrackView& v, float px,
+                                             float py, const TrackCell& cell, int q) {
+  unsigned int ok = __ballot_sync(kFull, cell.ok);
+  if constexpr (L >= 8) {
+    const int base = (int)(threadIdx.x & 31) & ~(L - 1);
+    constexpr unsigned int kGroup = (1u << L) - 1u;
+    bool on = ((ok >> base) & kGroup) != 0u;
+    const bool open = cell.open & !on;
+    if (__any_sync(kFull, open)) {  // a list of more than sixteen segments
+      bool hit = false;
+      if (open)
+        for (int i = 16 + q; i < cell.cnt && !hit; i += L)
+          hit = seg_hit(tr, v, v.list[cell.off + i], px, py);
+      on = on | (((__ballot_sync(kFull, hit) >> base) & kGroup) != 0u);
+    }
+    return on;
+  }
+  unsigned int todo = __ballot_sync(kFull, cell.open), taken;
+  if constexpr (L == 2) {
+    // a candidate's lanes 2 g, 2 g + 1: on the road if either is, open if both are
+    ok |= ((ok >> 1) & 0x55555555u) | ((ok << 1) & 0xAAAAAAAAu);
+    todo &= (todo >> 1) & 0x55555555u;
+  }
+  while (todo != 0u) {
+    const unsigned int got = settle_open(tr, v, px, py, cell, todo, &taken);
+    ok |= L == 2 ? got | (got << 1) : got;
+  }
+  return ((ok >> (threadIdx.x & 31)) & 1u) != 0u;
+}
+
 // Both stages; all 32 lanes of a warp call it together, `active` says which have a
 // position.
 __device__ __forceinline__ bool track_ok_warp(const DevTrack& tr, const TrackView& v, float px,
@@ -656,8 +715,8 @@ __device__ __forceinline__ void fma_word(const float4 kv, const float* z, int w,
 // is held, Sec. VII-B), so the first part of the chain is the same number at
 // every step: it is summed once per candidate (hc) and each step continues the
 // chain from it -- the same rounding as summing it every step.
-template <int KIND, int L, int C, bool KSMEM, bool TRAJ, bool NOISE, bool HELD, class P,
-          class KR>
+template <int KIND, int L, int C, bool KSMEM, bool TRAJ, bool NOISE, bool HELD,
+          bool PIPED = true, class P, class KR>
 __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety& safety,
                                          int wt, int n_eval,
                                          const float* xs, const float* uh, float sn, float cs,
@@ -784,6 +843,7 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
   // candidate per thread leaves free)
   constexpr int PREG = (PK && C == 1) ? 2 : 0;
   float4 kreg[PREG > 0 ? PREG : 1][PREG > 0 ? KP::NF / 2 : 1];
+  if constexpr (PREG == 0) kreg[0][0] = make_float4(0.f, 0.f, 0.f, 0.f);
   if constexpr (PREG > 0) {
 #pragma unroll
     for (int pp = 0; pp < PREG; ++pp)
@@ -800,7 +860,8 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
   // N = 1024 (16 lanes) 60 -> 30 us, N = 4096 (8) 76 -> 44, N = 16384 (2) 97 -> 80.
   constexpr int AHEAD = !NOISE ? 1 : (L > 1 ? L : (KIND != kCar && C == 1 ? 4 : 1));
   float ahead[AHEAD >= L ? AHEAD / L : 1][NX];
-  for (int t = 1; t <= H; ++t) {
+  // z <- K z, then the step's noise
+  const auto advance = [&](int t) {
     if constexpr (PK) {
       // z <- K z with the free rows in pairs (see KPair): per pair one chain of
       // packed FMAs, continuing from the held columns' share, over the free
@@ -991,6 +1052,8 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
         z[0][k] = v.x; z[0][k + 1] = v.y; z[0][k + 2] = v.z; z[0][k + 3] = v.w;
       }
     }
+  };
+  const auto perturb = [&](int t) {
     if constexpr (NOISE && AHEAD > 1) {
       // lane q of the group draws steps t + q, t + L + q, ..., and each step reads its
       // lane's normals
@@ -1016,34 +1079,85 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
       for (int c = 0; c < C; ++c)
         if (alive[c]) add_noise<NX>(a, d, slot[c], t, z[c]);
     }
-    bool any_alive = false;
+  };
+  const auto record = [&](int t) {
+    if constexpr (TRAJ) {
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      if constexpr (TRAJ) {
+      for (int c = 0; c < C; ++c)
         if (traj[c] != nullptr && alive[c]) {
 #pragma unroll
           for (int j = 0; j < N; ++j) traj[c][(size_t)t * N + j] = z[c][j];
         }
-      }
-      bool ok = box_ok<NX>(safety, z[c]);
-      if constexpr (B::TRACK) {
-        if (safety.has_track) {  // uniform over the grid
-          // every lane of the warp calls this (L = 1: the warp-wide test)
-          bool on_road;
-          if constexpr (L == 1)
-            on_road = track_ok_warp(safety.track, tv, z[c][0], z[c][1], alive[c] && ok);
-          else
-            on_road = track_ok<L>(safety.track, tv, z[c][0], z[c][1], q, alive[c] && ok);
-          ok = ok && on_road;
-        }
-      }
-      if (alive[c]) {
-        if (ok) ttv[c] = t;
-        else alive[c] = false;
-      }
-      any_alive = any_alive || alive[c];
     }
-    if (!__any_sync(kFull, any_alive)) break;
+  };
+  // PIPED, with a track: the test of step t runs beside the
+  // product of step t + 1.  Its loads (cell, list, segments) and their arithmetic form
+  // one long chain, and placed before the product in the same straight line of code
+  // they fill with its FMAs.  What remains after the product is the vote and the open
+  // positions (settle_open).  A tile whose last candidate leaves at step t has then
+  // computed step t + 1 for nothing.  Race car, H = 60, one warp per SM sub-partition:
+  // sixteen lanes (N = 1024) 25.7 -> 20.8 us, eight (N = 2048) 29.7 -> 22.8, two (N =
+  // 8192) 44.7 -> 35.3, one 64 -> 60, two candidates per thread 99 -> 88; two warps
+  // (N = 16384, two lanes) 57.0 -> 53.3.  Served batches and sorted tiles of two
+  // candidates per thread keep the pipes full without it (3 and 1 % slower piped).
+  constexpr bool PIPE = PIPED && B::TRACK && HELD && (KSMEM ? L <= 2 : L >= 8);
+  if (PIPE && safety.has_track) {
+    if constexpr (PIPE) {
+      advance(1);
+      for (int t = 1; t <= H; ++t) {
+        perturb(t);
+        record(t);
+        TrackCell cell[C];
+        float px[C], py[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          px[c] = z[c][0];
+          py[c] = z[c][1];
+          cell[c] = track_front<L>(safety.track, tv, px[c], py[c],
+                                   alive[c] & box_ok<NX>(safety, z[c]), q);
+        }
+        advance(t + 1);
+        bool any_alive = false;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+          const bool ok = track_settle<L>(safety.track, tv, px[c], py[c], cell[c], q);
+          if (alive[c]) {
+            if (ok) ttv[c] = t;
+            else alive[c] = false;
+          }
+          any_alive = any_alive || alive[c];
+        }
+        if (!__any_sync(kFull, any_alive)) break;
+      }
+    }
+  } else {
+    for (int t = 1; t <= H; ++t) {
+      advance(t);
+      perturb(t);
+      record(t);
+    bool any_alive = false;
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        bool ok = box_ok<NX>(safety, z[c]);
+        if constexpr (B::TRACK) {
+          if (safety.has_track) {  // uniform over the grid
+            // every lane of the warp calls this (L = 1: the warp-wide test)
+            bool on_road;
+            if constexpr (L == 1)
+              on_road = track_ok_warp(safety.track, tv, z[c][0], z[c][1], alive[c] && ok);
+            else
+              on_road = track_ok<L>(safety.track, tv, z[c][0], z[c][1], q, alive[c] && ok);
+            ok = ok && on_road;
+          }
+        }
+        if (alive[c]) {
+          if (ok) ttv[c] = t;
+          else alive[c] = false;
+        }
+        any_alive = any_alive || alive[c];
+      }
+      if (!__any_sync(kFull, any_alive)) break;
+    }
   }
 
 #pragma unroll
@@ -1352,7 +1466,8 @@ __global__ void __launch_bounds__(kMaxBlock) tick_kernel(const __grid_constant__
   const int wpb = blockDim.x >> 5;
   constexpr int PER_WARP = GPW * C;  // candidate slots per warp-tile
   const auto tile = [&](int wt, int cnt, const uint16_t* order, int base) {
-    run_tile<KIND, L, C, KSMEM, TRAJ, NOISE, !PARTIALS>(
+    // sorted tiles of two candidates per thread keep the pipes full without piping
+    run_tile<KIND, L, C, KSMEM, TRAJ, NOISE, !PARTIALS, !(UNITS && C == 2)>(
         a, dyn_of(a), a.safety, wt, cnt, xs, uh, sn, cs, kr, sK4, tv,
         &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec, order, base);
   };
