@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_const
   __shared__ float s_f[N][4];  // split of the lifting at x_t: a_j, b_1j, b_2j, b_3j
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  grid_dep_wait();
   if (fallback_not_needed(a)) return;
   const int n_eval = a.n_list ? *a.n_list : a.n_slots;
   const int H = a.horizon, ro_n = a.ro_n;
@@ -257,16 +258,17 @@ __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_const
       if (a.cost_out) a.cost_out[slot] = cost;
     }
   }
+  grid_dep_release();
   session_epilogue<NU, TickArgs, kFactBlock / 32>(a, best, n_safe, n_exec, uh, failed,
                                                   (unsigned int)n_active);
 }
 
 template <int KIND>
-static const void* factored_fn() {
-  return reinterpret_cast<const void*>(&factored_kernel<KIND>);
+static void (*factored_fn())(TickArgs) {
+  return &factored_kernel<KIND>;
 }
 
-static const void* pick_factored(int kind) {
+static void (*pick_factored(int kind))(TickArgs) {
   switch (kind) {
     case kBot: return factored_fn<kBot>();
     case kCar: return factored_fn<kCar>();
@@ -292,7 +294,7 @@ int compute_powers(int kind, const float* K, int H, float* out, cudaStream_t st)
 }
 
 int launch_factored(mpmi_session* s, TickArgs& a, cudaStream_t st, int n_hint) {
-  const void* fn = pick_factored(s->model->kind);
+  void (*const fn)(TickArgs) = pick_factored(s->model->kind);
   if (!fn) return fail(MPMI_E_UNSUPPORTED, "factored kernel not compiled for this basis");
   const size_t track = a.safety.has_track ? (size_t)a.safety.track.blob_bytes : 0;
   const size_t smem = track + (size_t)a.horizon * a.ro_n * sizeof(float4);
@@ -317,8 +319,7 @@ int launch_factored(mpmi_session* s, TickArgs& a, cudaStream_t st, int n_hint) {
   int grid = (n_work + wpb - 1) / wpb;
   if (grid > s->fact_grid) grid = s->fact_grid;
   if (grid < 1) grid = 1;
-  void* args[] = {&a};
-  const cudaError_t e = cudaLaunchKernel(fn, dim3(grid), dim3(32 * wpb), args, smem, st);
+  const cudaError_t e = launch_dependent(fn, grid, 32 * wpb, smem, st, a);
   if (e != cudaSuccess)
     return fail(MPMI_E_CUDA, std::string("factored kernel launch: ") + cudaGetErrorString(e));
   return MPMI_OK;

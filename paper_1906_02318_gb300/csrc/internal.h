@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "mpmi.h"
@@ -87,8 +88,8 @@ struct TickArgs {
   int ro_idx[MPMI_MAX_NX];
   // test hook: stage nothing, so the bounded staging wait runs out
   int withhold_staging;
-  // launched as a programmatic dependent of the previous kernel on the stream
-  // (a screened tick's chain): wait for it before reading anything
+  // a launch of a screened tick's chain, which the launch before it lets start early:
+  // wait for that one before reading anything, then let the next one start
   int chained;
   // zero-copy host ticks: after the result, the decoding block stores seq here
   // (pinned host memory) behind a system-scope fence
@@ -179,6 +180,7 @@ struct mpmi_session {
   // select_input returned on the completion word while the kernel may still be
   // resetting the reduction record: the next launch waits for `done` first
   bool tail_pending = false;
+  unsigned long long tail_stream = ~0ull;  // that kernel's stream (cudaStreamGetId)
   cudaEvent_t done = nullptr;
   bool in_flight = false;
   float noise_sigma[MPMI_MAX_NX] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -223,6 +225,28 @@ struct DeviceGuard {
     if (changed) cudaSetDevice(prev);
   }
 };
+
+#ifdef __CUDACC__
+// Launches a kernel as a programmatic dependent of the one before it on the stream: it
+// may start while that one still runs, and calls grid_dep_wait before it touches
+// anything another kernel may write.  (After a kernel that never calls
+// grid_dep_release, or after a copy, it starts when that has ended.)
+template <class... KA, class... A>
+static cudaError_t launch_dependent(void (*fn)(KA...), int grid, int block, size_t smem,
+                                    cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fn, std::forward<A>(args)...);
+}
+#endif
 
 // tick launch helpers shared by the API and the screener (mpmi_api.cu)
 TickArgs make_tick_args(const mpmi_session* s, uint64_t tick);

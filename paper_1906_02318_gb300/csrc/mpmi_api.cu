@@ -280,6 +280,7 @@ int host_tick_begin(mpmi_session* s) {
 // After a host tick's launches on st: the event select_input falls back to.
 int host_tick_end(mpmi_session* s, cudaStream_t st) {
   MPMI_CUDA(cudaEventRecord(s->done, st), "cudaEventRecord");
+  MPMI_CUDA(cudaStreamGetId(st, &s->tail_stream), "cudaStreamGetId");
   s->in_flight = true;
   return MPMI_OK;
 }
@@ -292,8 +293,12 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
     if (rc != MPMI_OK) return rc;
   }
   if (s->tail_pending) {
-    // the previous host tick's kernel may still be finishing: order behind it
-    const cudaError_t e = cudaStreamWaitEvent(st, s->done, 0);
+    // the previous host tick's kernel may still be finishing: order behind it (on its
+    // own stream the launch follows it anyway)
+    unsigned long long id = 0;
+    cudaError_t e = cudaStreamGetId(st, &id);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamGetId");
+    if (id != s->tail_stream) e = cudaStreamWaitEvent(st, s->done, 0);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamWaitEvent");
     s->tail_pending = false;
   }

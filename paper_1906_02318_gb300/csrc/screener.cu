@@ -109,6 +109,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(const float* __r
   float *sW2 = sm + S::W2, *sH1 = sm + S::H1, *sG1 = sm + S::G1, *sD2 = sm + S::D2,
         *sW1 = sm + S::W1, *sb1 = sm + S::B1, *sb2 = sm + S::B2, *sw3 = sm + S::W3,
         *sF = sm + S::F, *red = sm + S::RED;
+  grid_dep_wait();     // the weights of the step before
   grid_dep_release();  // the reduction may launch now; it waits for this kernel
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int jg = tid & 15, sg = tid >> 4;  // 16 column groups x 16 sample groups
@@ -350,6 +351,7 @@ __global__ void __launch_bounds__(kRedSlices * kRedParams) reduce_grad(const flo
   const int x = threadIdx.x % kRedParams, y = threadIdx.x / kRedParams;
   const int i = blockIdx.x * kRedParams + x;
   grid_dep_wait();
+  grid_dep_release();
   float g = 0.f;
   if (i <= kP) {
 #pragma unroll 16
@@ -906,15 +908,16 @@ __global__ void __launch_bounds__(kScoreThreads) screen_score(TickArgs a, Featur
   __shared__ float s_feat[12];
   __shared__ uint64_t s_bar;
   __shared__ uint32_t s_tmem;
-  grid_dep_release();  // the compaction may launch now; it waits for this kernel
   for (int i = threadIdx.x; i < kBins; i += blockDim.x) {
     s_hist[i] = 0;
     s_hsafe[i] = 0;
   }
   ScoreCtx c;
   WeightRegs wr;
-  weights_load(w, wr);  // in flight while the accumulator and the features are prepared
   score_begin(s_score, &s_bar, &s_tmem, &c);
+  grid_dep_wait();      // the inputs, and the last screened tick's use of the scratch
+  grid_dep_release();   // the compaction may launch now; it waits for this kernel
+  weights_load(w, wr);  // in flight while the features are prepared
   block_tick_features(fs, a.x_t, s_feat);  // ends with __syncthreads
   weights_store(wr, s_score);
   float uh[2] = {__double2float_rn(a.u_h[0]), __double2float_rn(a.u_h[1])};
@@ -971,8 +974,9 @@ __global__ void __launch_bounds__(kScoreThreads) screen_score(TickArgs a, Featur
 __global__ void __launch_bounds__(128) screen_cost(TickArgs a, int k, unsigned int* keys,
                                                   ScreenScratch* ss) {
   __shared__ unsigned int s_hist[kBins];
-  grid_dep_release();  // the compaction may launch now; it waits for this kernel
   for (int i = threadIdx.x; i < kBins; i += blockDim.x) s_hist[i] = 0;
+  grid_dep_wait();     // the inputs, and the last screened tick's use of the scratch
+  grid_dep_release();  // the compaction may launch now; it waits for this kernel
   __syncthreads();
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5;
@@ -1108,28 +1112,17 @@ static int gradients(mpmi_screener* s, const float* feats, const float* target, 
   const int spt = train_spt(B, s->ctx->sm_count);
   const int tiles = (B + 16 * spt - 1) / (16 * spt);
   const int blocks = tiles < s->n_part ? tiles : s->n_part;
-  if (spt == 4)
-    train_tiles<4><<<blocks, kTrainThreads, TrainSmem<4>::BYTES, st>>>(s->params, feats, target, B,
-                                                                       s->part);
-  else if (spt == 2)
-    train_tiles<2><<<blocks, kTrainThreads, TrainSmem<2>::BYTES, st>>>(s->params, feats, target, B,
-                                                                       s->part);
-  else
-    train_tiles<1><<<blocks, kTrainThreads, TrainSmem<1>::BYTES, st>>>(s->params, feats, target, B,
-                                                                       s->part);
-  SCR_CUDA(cudaGetLastError(), "train_tiles launch");
-  // a programmatic dependent: it may launch while the tiles run and waits for them
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((kP + 1 + kRedParams - 1) / kRedParams));
-  cfg.blockDim = dim3(kRedSlices * kRedParams);
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  SCR_CUDA(cudaLaunchKernelEx(&cfg, reduce_grad, (const float*)s->part, blocks, B, grad, loss,
-                              s->params, s->adam_m, s->adam_v, lr, c1, c2),
+  const auto run = [&](auto fn, int smem) {
+    return launch_dependent(fn, blocks, kTrainThreads, (size_t)smem, st, (const float*)s->params,
+                            feats, target, B, s->part);
+  };
+  SCR_CUDA(spt == 4   ? run(train_tiles<4>, TrainSmem<4>::BYTES)
+           : spt == 2 ? run(train_tiles<2>, TrainSmem<2>::BYTES)
+                      : run(train_tiles<1>, TrainSmem<1>::BYTES),
+           "train_tiles launch");
+  SCR_CUDA(launch_dependent(reduce_grad, (kP + 1 + kRedParams - 1) / kRedParams,
+                            kRedSlices * kRedParams, 0, st, (const float*)s->part, blocks, B, grad,
+                            loss, s->params, s->adam_m, s->adam_v, lr, c1, c2),
            "reduce_grad launch");
   return MPMI_OK;
 }
@@ -1169,34 +1162,23 @@ static int screened_chain(mpmi_session* session, mpmi_screener* s, const TickArg
   if (tau > 0.f) {
     const int tiles = (session->n_slots + kTileRows - 1) / kTileRows;
     const int blocks = tiles < 2 * s->ctx->sm_count ? tiles : 2 * s->ctx->sm_count;
-    screen_score<<<blocks, kScoreThreads, kScoreSmem, st>>>(sa, feature_src(s), s->infer, tau,
-                                                            k, m, s->keys, s->ss);
+    SCR_CUDA(launch_dependent(screen_score, blocks, kScoreThreads, kScoreSmem, st, sa,
+                              feature_src(s), (const InferW*)s->infer, tau, (int)k, (int)m, s->keys,
+                              s->ss),
+             "screen_score launch");
   } else {
     const int tiles = (session->n_slots + 15) / 16;
     int blocks = (tiles + 3) / 4;
     if (blocks > 2 * s->ctx->sm_count) blocks = 2 * s->ctx->sm_count;
-    screen_cost<<<blocks, 128, 0, st>>>(sa, k, s->keys, s->ss);
+    SCR_CUDA(launch_dependent(screen_cost, blocks, 128, 0, st, sa, (int)k, s->keys, s->ss),
+             "screen_cost launch");
   }
   if (s->timing) SCR_CUDA(cudaEventRecord(s->ev[1], st), "cudaEventRecord");
   int cb = (session->n_slots + 255) / 256;
   if (cb > 4 * s->ctx->sm_count) cb = 4 * s->ctx->sm_count;
-  {
-    // the compaction, the rollout and the fallback run as programmatic
-    // dependents: each may launch while its predecessor runs and waits for it
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)cb);
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    SCR_CUDA(cudaLaunchKernelEx(&cfg, screen_compact, (const unsigned int*)s->keys,
-                                (int)session->n_slots, s->ss, s->list),
-             "screen_compact launch");
-  }
-  SCR_CUDA(cudaGetLastError(), "screen launches");
+  SCR_CUDA(launch_dependent(screen_compact, cb, 256, 0, st, (const unsigned int*)s->keys,
+                            (int)session->n_slots, s->ss, s->list),
+           "screen_compact launch");
   if (s->timing) SCR_CUDA(cudaEventRecord(s->ev[2], st), "cudaEventRecord");
   // exact rollout on the kept slots (their number is known only on the device)
   TickArgs r = a;
@@ -1467,6 +1449,7 @@ int mpmi_evaluate_screened_host(mpmi_session* session, mpmi_screener* s, const d
   if ((rc = screened_chain(session, s, a, k, tau, m, nullptr, nullptr, st)) != MPMI_OK) {
     // launches queued before the failing one may still run: later launches and
     // closing the session wait for them
+    session->tail_stream = ~0ull;  // whatever the next launch's stream, order it by the event
     if (cudaEventRecord(session->done, st) == cudaSuccess) session->tail_pending = true;
     return rc;
   }

@@ -155,6 +155,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_tick_kernel(const __grid_con
   // writes the other slot while a slower one still reads this one
   __shared__ int s_fail[kTcHalves][2];
 
+  grid_dep_wait();
   if (fallback_not_needed(a)) return;
   const int n_eval = a.n_list ? *a.n_list : a.n_slots;
   const int H = a.horizon;
@@ -394,6 +395,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_tick_kernel(const __grid_con
       if (a.cost_out) a.cost_out[slot] = cost;
     }
   }
+  grid_dep_release();
   tc_fence_before();
   failed = __syncthreads_or(failed) != 0;  // a half's failed wait flags the whole block
   tc_fence_after();
@@ -405,8 +407,8 @@ __global__ void __launch_bounds__(kTcThreads, 2) tc_tick_kernel(const __grid_con
 }
 
 template <bool TRAJ>
-static const void* tc_fn() {
-  return reinterpret_cast<const void*>(&tc_tick_kernel<kCar, TRAJ>);
+static void (*tc_fn())(TickArgs) {
+  return &tc_tick_kernel<kCar, TRAJ>;
 }
 
 // The tensor-core rollout's CTAs per SM and the dynamic shared memory that keeps
@@ -443,7 +445,8 @@ static int tc_resident(const void* fn, size_t need, int device, size_t* smem_out
 int launch_tensor(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, int n_hint) {
   if (s->model->kind != kCar)
     return fail(MPMI_E_UNSUPPORTED, "the tensor-core rollout is compiled for the race car");
-  const void* fn = traj ? tc_fn<true>() : tc_fn<false>();
+  void (*const run)(TickArgs) = traj ? tc_fn<true>() : tc_fn<false>();
+  const void* fn = reinterpret_cast<const void*>(run);
   const size_t smem =
       kTcFixedSmem + (a.safety.has_track ? (size_t)a.safety.track.blob_bytes : 0);
   const int t = traj ? 1 : 0;
@@ -466,9 +469,7 @@ int launch_tensor(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, int 
   int grid = (n_work + kTcM - 1) / kTcM;
   if (grid > s->tc_grid[t]) grid = s->tc_grid[t];
   if (grid < 1) grid = 1;
-  void* args[] = {&a};
-  const cudaError_t e =
-      cudaLaunchKernel(fn, dim3(grid), dim3(kTcThreads), args, s->tc_req[t], st);
+  const cudaError_t e = launch_dependent(run, grid, kTcThreads, s->tc_req[t], st, a);
   if (e != cudaSuccess)
     return fail(MPMI_E_CUDA, std::string("tensor-core tick launch: ") + cudaGetErrorString(e));
   return MPMI_OK;

@@ -1,0 +1,112 @@
+"""Launches that may start before the previous kernel on the stream ends still read what
+it wrote: inputs updated between ticks, results chained from tick to tick, several
+streams, and graph replays."""
+import numpy as np
+import pytest
+
+from workloads import data
+
+from parity import bot_env, car_env, gpu_model
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def setup():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1906_02318_gb300 import build, mpmi
+    build.build()
+    ctx = mpmi.Context(0)
+    envs = dict(bot=bot_env(), car=car_env())
+    return mpmi, ctx, {k: (e, gpu_model(mpmi, ctx, e)) for k, e in envs.items()}
+
+
+def _case(lib, ctx, envs, which, N, rollout):
+    import torch
+    env, model = envs[which]
+    s = lib.Session(ctx, model, N, 40, env.lo, env.hi, seed=3)
+    s.set_rollout(rollout)
+    x = (np.array([0.05, 0.1, 0.2, -0.1]) if which == "bot"
+         else data.car_start_state(env.track, vx=12.0))
+    u = data.to_f32_exact(data.user_input_once(2, env.lo, env.hi))
+    dev = lambda a: torch.tensor(a, dtype=torch.float64, device="cuda")  # noqa: E731
+    return s, dev(x), dev(u)
+
+
+CASES = [("bot", 900, "full"), ("bot", 70000, "full"), ("bot", 3000, "factored"),
+         ("car", 900, "full"), ("car", 16384, "full"), ("car", 66000, "full"),
+         ("car", 5000, "tensor"), ("car", 5000, "factored")]
+
+
+def _step(lib, s, x, u, res, t):
+    """One tick, then a torch kernel that moves the state by the tick's own result."""
+    lib.evaluate_candidates_device(s, x, u, res, tick=t)
+    u_r = res[:8 * s.nu].view(dtype=x.dtype)
+    x[1:1 + s.nu] += 0.01 * u_r
+
+
+@pytest.mark.parametrize("which,N,rollout", CASES)
+def test_back_to_back_ticks_see_each_other(setup, which, N, rollout):
+    import torch
+    lib, ctx, envs = setup
+    out = []
+    for wait in (True, False):
+        s, x, u = _case(lib, ctx, envs, which, N, rollout)
+        res = torch.zeros((30, lib.RESULT_BYTES), dtype=torch.uint8, device="cuda")
+        for t in range(30):
+            _step(lib, s, x, u, res[t], t)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        out.append((res.cpu().numpy(), x.cpu().numpy()))
+        s.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("which,N,rollout", CASES)
+def test_captured_ticks_replay(setup, which, N, rollout):
+    import torch
+    lib, ctx, envs = setup
+    s, x, u = _case(lib, ctx, envs, which, N, rollout)
+    x0 = x.clone()
+    res = torch.zeros((4, lib.RESULT_BYTES), dtype=torch.uint8, device="cuda")
+
+    def run():
+        x.copy_(x0)
+        for t in range(4):
+            _step(lib, s, x, u, res[t], t)
+
+    run()
+    torch.cuda.synchronize()
+    want = res.cpu().numpy().copy()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        run()
+    for _ in range(3):
+        res.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(res.cpu().numpy(), want)
+    s.close()
+
+
+def test_host_ticks_alternate_streams(setup):
+    """A host tick is ordered behind the last one's kernel whichever stream it takes."""
+    import torch
+    lib, ctx, envs = setup
+    env, model = envs["bot"]
+    streams = [torch.cuda.current_stream(), torch.cuda.Stream(), torch.cuda.Stream()]
+    out = []
+    for pick in (lambda t: 0, lambda t: t % 3, lambda t: (t // 2) % 3):
+        s = lib.Session(ctx, model, 4096, 40, env.lo, env.hi, seed=8)
+        got = []
+        for t in range(40):
+            lib.evaluate_candidates(s, [0.05, 0.01 * t, 0.0, 0.0], [0.3], tick=t,
+                                    stream=streams[pick(t)])
+            r = lib.select_input(s)
+            got.append((r["index"], r["n_safe"], r["executed_steps"], float(r["u_r"][0])))
+        s.close()
+        out.append(got)
+    assert out[0] == out[1] == out[2]
