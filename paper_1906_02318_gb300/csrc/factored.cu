@@ -56,36 +56,95 @@ __global__ void __launch_bounds__(256) powers_kernel(const float* K, int H, floa
   }
 }
 
+// Steps t0 + 1 .. t0 + 32 of a candidate with input monomials p, one per lane: the lane
+// of the first that violates the safety set, or 32.  RO read-outs (0: ro_n of them).
+// Only the first violation counts, so open positions (settle_open) are settled in the
+// order of their steps, and none after a step that is known to violate.
+template <int KIND, int RO>
+__device__ __forceinline__ int first_violation(const DevTrack& tr, const TrackView& tv, bool track,
+                                               const float4* V, int ro_n, int H, int t0,
+                                               const float* lo, const float* hi, float4 p) {
+  constexpr int NX = BasisTraits<KIND>::NX, NP = BasisTraits<KIND>::NP;
+  const int lane = threadIdx.x & 31, t = t0 + lane + 1;
+  const int n = RO ? RO : ro_n;
+  bool ok = true;
+  float px = 0.f, py = 0.f;
+  if (t <= H) {
+    const float4* Vt = V + (t - 1) * n;
+#pragma unroll
+    for (int r = 0; r < (RO ? RO : NX); ++r) {
+      if (RO || r < n) {
+        const float4 w = Vt[r];
+        float v = __fmaf_rn(p.x, w.y, w.x);
+        if constexpr (NP > 1) v = __fmaf_rn(p.y, w.z, v);
+        if constexpr (NP > 2) v = __fmaf_rn(p.z, w.w, v);
+        ok = ok & (v > lo[r]) & (v < hi[r]);
+        if (r == 0) px = v;
+        if (r == 1) py = v;
+      }
+    }
+  }
+  unsigned int bad;
+  if (BasisTraits<KIND>::TRACK && track) {
+    const TrackCell cell = track_cell(tr, tv, px, py, ok && t <= H);
+    ok = ok && (cell.ok || cell.open || t > H);
+    bad = __ballot_sync(kFull, !ok);
+    unsigned int todo = __ballot_sync(kFull, cell.open), taken;
+    if (bad != 0u) todo &= (bad & (0u - bad)) - 1u;  // before the first violation
+    while (todo != 0u) {
+      const unsigned int got = settle_open(tr, tv, px, py, cell, todo, &taken);
+      if ((taken & ~got) != 0u) {  // an earlier violation than any left open
+        bad |= taken & ~got;
+        break;
+      }
+    }
+  } else {
+    bad = __ballot_sync(kFull, !ok);
+  }
+  return bad != 0u ? __ffs(bad) - 1 : 32;
+}
+
 // One tick in the factorised form.  Dynamic shared memory: [track grid (race
 // car)] [V: H x ro_n float4, (a, b_1, b_2, b_3) coefficients per read-out].
-// Bound: issue (57 % of the slots; about 190 instructions per 32 steps of a candidate,
-// the track test most of them), with a quarter of the warps' time at the barriers of
-// the prologue and the reduction.  GB300, race car, N = 30001, H = 100: 30.0 us, 56.7
-// with 760 blocks of 128 threads that tested every listed segment of every step.
+// One block per SM.  A block draws up to a thread's candidate each, then its warps take
+// the drawn candidates from a counter and test 32 steps of one at a time (the read-outs
+// of different steps do not depend on each other; lane l: step t0 + l + 1), until the
+// first violation.  Bound: issue, about 190 instructions per 32 steps, the track test
+// most of them.  GB300, race car, N = 30001, H = 100: 25.6 us; 56.7 with 760 blocks of
+// 128 threads that each staged the grid and built V, gave some warps two tiles and
+// others one, and tested every listed segment of every step; 28.0 with equal tiles per
+// warp and one feature per lane in the prologue (10k cycles of a 32-way switch).
 template <int KIND>
 __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_constant__ TickArgs a) {
   using B = BasisTraits<KIND>;
   constexpr int N = B::N, NX = B::NX, NU = B::NU, NP = B::NP;
   constexpr int ANG = (KIND == kBot) ? 0 : ((KIND == kCar) ? 2 : -1);
   extern __shared__ uint4 s_dyn[];
-  __shared__ float s_f[N][4];  // split of the lifting at x_t: a_j, b_1j, b_2j, b_3j
+  __shared__ float4 s_f[N];  // split of the lifting at x_t: a_j, b_1j, b_2j, b_3j
+  __shared__ float4 s_cand[kFactBlock];  // drawn candidates: monomials (up to 3), cost
+  __shared__ int s_ttv[kFactBlock];
+  __shared__ int s_next;
+  __shared__ uint64_t s_bar;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  grid_dep_wait();
+  // a launch over every slot that is sure to run stages the session's constants while
+  // the kernel before it ends; the others look at that kernel's results first
+  const bool sure = a.skip_if_safe == nullptr && a.n_list == nullptr;
+  if (!sure) grid_dep_wait();
   if (fallback_not_needed(a)) return;
   const int n_eval = a.n_list ? *a.n_list : a.n_slots;
   const int H = a.horizon, ro_n = a.ro_n;
-  // every warp takes an equal share of the candidates, at most 32 at a time; the
-  // blocks that a short device-side list leaves without a share return at once
+  // equal shares of the candidates, at least one per warp; the blocks that a short
+  // device-side list leaves without a share return at once
   const int wpb = blockDim.x >> 5;
-  const int warps = (int)gridDim.x * wpb;
-  const int tile = max(1, min(32, (n_eval + warps - 1) / warps));
-  const int n_wtiles = (n_eval + tile - 1) / tile;
-  const int n_active = max(1, min((int)gridDim.x, (n_wtiles + wpb - 1) / wpb));
-  if ((int)blockIdx.x >= n_active) return;
+  const int share = max(wpb, (n_eval + (int)gridDim.x - 1) / (int)gridDim.x);
+  const int n_active = max(1, (n_eval + share - 1) / share);
+  if ((int)blockIdx.x >= n_active) {
+    if (sure) grid_dep_wait();
+    return;
+  }
 
   // the track grid arrives by bulk copy while the table V is built
-  __shared__ uint64_t s_bar;
   const bool track_on = B::TRACK && a.safety.has_track;
   if (track_on) {
     if (tid == 0) bar_init(&s_bar);
@@ -107,47 +166,66 @@ __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_const
     }
   }
   float4* V = reinterpret_cast<float4*>(s_dyn + track_words);
-
-  float xs[NX], uh[NU];
+  // this thread's first row C K^t, in flight during the wait and the lifting
+  constexpr int N4 = N % 4 == 0 ? N / 4 : 0;
+  const auto row_of = [&](int e) {
+    const int t = e / ro_n, r = e - t * ro_n;
+    return a.ck + ((size_t)t * NX + a.ro_idx[r]) * N;
+  };
+  float4 p4[N4 ? N4 : 1];
+  if (N4 && tid < H * ro_n) {
+    const float4* row = reinterpret_cast<const float4*>(row_of(tid));
 #pragma unroll
-  for (int j = 0; j < NX; ++j) xs[j] = __double2float_rn(a.x_t[j]);
+    for (int j = 0; j < N4; ++j) p4[j] = __ldg(row + j);
+  }
+  if (sure) grid_dep_wait();
+
+  float uh[NU];
 #pragma unroll
   for (int j = 0; j < NU; ++j) uh[j] = __double2float_rn(a.u_h[j]);
-  float sn = 0.f, cs = 1.f;
-  if constexpr (ANG >= 0) sincosf(xs[ANG], &sn, &cs);
-  for (int j = tid; j < N; j += blockDim.x) {
-    float av, bv[kMaxP];
-    feature_split<float>(KIND, j, xs, sn, cs, &av, bv);
-    s_f[j][0] = av;
+  if (warp == 0) {
+    // every feature in straight-line code by each lane of one warp (one feature per
+    // lane would take the switch's 32 ways one after the other)
+    float xs[NX], sn = 0.f, cs = 1.f;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) s_f[j][1 + k] = k < NP ? bv[k] : 0.f;
+    for (int j = 0; j < NX; ++j) xs[j] = __double2float_rn(a.x_t[j]);
+    if constexpr (ANG >= 0) sincosf(xs[ANG], &sn, &cs);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      float av, bv[kMaxP];
+      feature_split<float>(KIND, j, xs, sn, cs, &av, bv);
+      if (lane == (j & 31))
+        s_f[j] = make_float4(av, bv[0], NP > 1 ? bv[1] : 0.f, NP > 2 ? bv[2] : 0.f);
+    }
   }
   __syncthreads();
   // V[t][r] = (P_t row ro_idx[r]) . (a, b_1, b_2, b_3)
   for (int e = tid; e < H * ro_n; e += blockDim.x) {
-    const int t = e / ro_n, r = e - t * ro_n;
-    const float* prow = a.ck + ((size_t)t * NX + a.ro_idx[r]) * N;
     float v0 = 0.f, v1 = 0.f, v2 = 0.f, v3 = 0.f;
     const auto add = [&](int j, float pj) {
-      v0 = __fmaf_rn(pj, s_f[j][0], v0);
-      v1 = __fmaf_rn(pj, s_f[j][1], v1);
-      v2 = __fmaf_rn(pj, s_f[j][2], v2);
-      v3 = __fmaf_rn(pj, s_f[j][3], v3);
+      const float4 f = s_f[j];
+      v0 = __fmaf_rn(pj, f.x, v0);
+      v1 = __fmaf_rn(pj, f.y, v1);
+      v2 = __fmaf_rn(pj, f.z, v2);
+      v3 = __fmaf_rn(pj, f.w, v3);
     };
-    if constexpr (N % 4 == 0) {  // rows of whole float4s: all of a row's loads in flight
-      float4 p4[N / 4];
+    if constexpr (N4 > 0) {  // rows of whole float4s: all of a row's loads in flight
+      if (e != tid) {
+        const float4* row = reinterpret_cast<const float4*>(row_of(e));
 #pragma unroll
-      for (int j = 0; j < N / 4; ++j) p4[j] = __ldg(reinterpret_cast<const float4*>(prow) + j);
+        for (int j = 0; j < N4; ++j) p4[j] = __ldg(row + j);
+      }
 #pragma unroll
-      for (int j = 0; j < N / 4; ++j) {
+      for (int j = 0; j < N4; ++j) {
         add(4 * j, p4[j].x);
         add(4 * j + 1, p4[j].y);
         add(4 * j + 2, p4[j].z);
         add(4 * j + 3, p4[j].w);
       }
     } else {
+      const float* row = row_of(e);
 #pragma unroll
-      for (int j = 0; j < N; ++j) add(j, __ldg(prow + j));
+      for (int j = 0; j < N; ++j) add(j, __ldg(row + j));
     }
     V[e] = make_float4(v0, v1, v2, v3);
   }
@@ -156,8 +234,6 @@ __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_const
     bool ok = bar_wait(&s_bar, 0);
     if (!ok) ok = bar_wait(&s_bar, 0);
     failed = __syncthreads_or(!ok) != 0;
-  } else {
-    __syncthreads();
   }
 
   // bounds of the read-out coordinates, in registers
@@ -167,94 +243,63 @@ __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_const
     lo[r] = r < ro_n ? a.safety.lo[a.ro_idx[r]] : -INFINITY;
     hi[r] = r < ro_n ? a.safety.hi[a.ro_idx[r]] : INFINITY;
   }
-  const bool track = B::TRACK && a.safety.has_track;  // read-outs 0, 1 are the position
 
   unsigned long long best = ~0ull;
   unsigned int n_safe = 0, n_exec = 0;
-  // Time-parallel: the read-outs of different steps do not depend on each other,
-  // so a warp takes its candidates one after the other and tests 32 steps of a
-  // candidate at once (lane l: step t0 + l + 1).  Only the first violation counts, so
-  // open positions (settle_open) are settled in the order of their steps, and none
-  // after a step that is known to violate.
-  for (int wt = failed ? n_wtiles : (int)blockIdx.x * wpb + warp; wt < n_wtiles; wt += warps) {
-    // lanes 0 .. tile - 1 draw and score one candidate each
-    const int pos = wt * tile + lane;
-    const int count = min(tile, n_eval - wt * tile);
-    const bool valid = lane < count;
-    const int slot = (valid && a.slot_list) ? a.slot_list[pos] : pos;
-    float xi[NU];
-    if (valid) {
-      candidate_value<NU>(a, slot, uh, xi);
-    } else {
-#pragma unroll
-      for (int j = 0; j < NU; ++j) xi[j] = uh[j];
-    }
+  const int first = (int)blockIdx.x * share;
+  const int end = failed ? first : min(first + share, n_eval);
+  for (int base = first; base < end; base += (int)blockDim.x) {
+    const int cnt = min((int)blockDim.x, end - base);
+    int slot = 0;
     float cost = 0.f;
+    if (tid < cnt) {
+      slot = a.slot_list ? a.slot_list[base + tid] : base + tid;
+      float xi[NU], p[NP];
+      candidate_value<NU>(a, slot, uh, xi);
 #pragma unroll
-    for (int j = 0; j < NU; ++j) {
-      const float d = __fsub_rn(xi[j], uh[j]);
-      cost = __fmaf_rn(d, d, cost);
+      for (int j = 0; j < NU; ++j) {
+        const float d = __fsub_rn(xi[j], uh[j]);
+        cost = __fmaf_rn(d, d, cost);
+      }
+      monomials32<KIND>(xi, p);
+      s_cand[tid] = make_float4(p[0], NP > 1 ? p[NP > 1 ? 1 : 0] : 0.f,
+                                NP > 2 ? p[NP > 2 ? 2 : 0] : 0.f, cost);
     }
-    float p[NP];
-    monomials32<KIND>(xi, p);
-    int my_ttv = 0;
-    for (int c = 0; c < count; ++c) {
-      float pc[NP];
-#pragma unroll
-      for (int k = 0; k < NP; ++k) pc[k] = __shfl_sync(kFull, p[k], c);
+    if (tid == 0) s_next = wpb;  // the warps' first candidates are 0 .. wpb - 1
+    __syncthreads();             // also: V is written
+    int c = warp;
+    while (c < cnt) {
+      int next = 0;
+      if (lane == 0) next = atomicAdd(&s_next, 1);
+      const float4 p = s_cand[c];
       int ttv = H;
       for (int t0 = 0; t0 < H; t0 += 32) {
-        const int t = t0 + lane + 1;
-        bool ok = true;
-        float px = 0.f, py = 0.f;
-        if (t <= H) {
-          const float4* Vt = V + (t - 1) * ro_n;
-#pragma unroll
-          for (int r = 0; r < NX; ++r) {
-            if (r < ro_n) {
-              const float4 w = Vt[r];
-              float v = __fmaf_rn(pc[0], w.y, w.x);
-              if constexpr (NP > 1) v = __fmaf_rn(pc[1], w.z, v);
-              if constexpr (NP > 2) v = __fmaf_rn(pc[2], w.w, v);
-              ok = ok && (v > lo[r]) && (v < hi[r]);
-              if (r == 0) px = v;
-              if (r == 1) py = v;
-            }
-          }
-        }
-        unsigned int bad;
-        if (B::TRACK && track) {
-          const TrackCell cell = track_cell(a.safety.track, tv, px, py, ok && t <= H);
-          ok = ok && (cell.ok || cell.open || t > H);
-          bad = __ballot_sync(kFull, !ok);
-          unsigned int todo = __ballot_sync(kFull, cell.open), taken;
-          if (bad != 0u) todo &= (bad & (0u - bad)) - 1u;  // before the first violation
-          while (todo != 0u) {
-            const unsigned int got =
-                settle_open(a.safety.track, tv, px, py, cell, todo, &taken);
-            if ((taken & ~got) != 0u) {  // an earlier violation than any left open
-              bad |= taken & ~got;
-              break;
-            }
-          }
-        } else {
-          bad = __ballot_sync(kFull, !ok);
-        }
-        if (bad != 0u) {
-          ttv = t0 + __ffs(bad) - 1;
+        // the usual numbers of read-outs in straight-line code: position and speed bound
+        // (race car), two bounded coordinates (balance bot)
+        constexpr int RO = KIND == kCar ? 3 : (NX >= 2 ? 2 : 0);
+        int at;
+        if (RO > 0 && ro_n == RO)
+          at = first_violation<KIND, RO>(a.safety.track, tv, track_on, V, RO, H, t0, lo, hi, p);
+        else
+          at = first_violation<KIND, 0>(a.safety.track, tv, track_on, V, ro_n, H, t0, lo, hi, p);
+        if (at < 32) {
+          ttv = t0 + at;
           break;
         }
       }
-      if (lane == c) my_ttv = ttv;
+      if (lane == 0) s_ttv[c] = ttv;
+      c = __shfl_sync(kFull, next, 0);
     }
-    if (valid) {
-      const unsigned long long key = ((unsigned long long)(H - my_ttv) << 55) |
+    __syncthreads();
+    if (tid < cnt) {
+      const int ttv = s_ttv[tid];
+      const unsigned long long key = ((unsigned long long)(H - ttv) << 55) |
                                      ((unsigned long long)__float_as_uint(cost) << 23) |
                                      (unsigned long long)slot;
       best = key < best ? key : best;
-      n_exec += (unsigned int)min(my_ttv + 1, H);
-      n_safe += my_ttv == H;
-      if (a.ttv_out) a.ttv_out[slot] = my_ttv;
+      n_exec += (unsigned int)min(ttv + 1, H);
+      n_safe += ttv == H;
+      if (a.ttv_out) a.ttv_out[slot] = ttv;
       if (a.cost_out) a.cost_out[slot] = cost;
     }
   }
