@@ -285,6 +285,18 @@ static std::vector<ServeKernel> serve_shapes(int kind) {
   return {};
 }
 
+// The shape an untuned server takes for batches of at least kLargeBatch slots per SM: two
+// race cars per thread, so that a word of K from shared memory, which bounds the one-lane
+// step, serves two predictions, in blocks of 256.  Race cars, N and H as in plan_batch,
+// submit to collect, one candidate per thread against two: 12 sessions (fewer slots than
+// that) 460 against 425 us alone but 513 against 564 with balance bots beside them, 16
+// sessions 604 against 529, 24 698 against 616, 60 1853 against 1575.  The balance bot
+// keeps K in registers and gains nothing.
+constexpr int kLargeBatch = 1200;
+static ServeKernel large_serve(int kind) {
+  return kind == kCar ? make_serve<kCar, 1, 2, true>() : ServeKernel{};
+}
+
 // Dynamic shared memory of a shape: K, the track grid, and a sorted unit.
 static size_t serve_smem(const ServeKernel& k, const DevSafety& safety) {
   return k.k_smem + (safety.has_track ? (size_t)safety.track.blob_bytes : 0) +
@@ -302,6 +314,16 @@ static ServeKernel pick_serve(int kind) {
 constexpr int kServeBuffers = 5;                      // batch buffers
 constexpr int kServeMaxInFlight = kServeBuffers - 1;  // one is always free for staging
 
+namespace mpmi {
+// A launch shape of the server with its captured graphs, one per batch buffer.
+struct ServeShape {
+  ServeKernel kern;
+  int grid = 0, block = 128;
+  size_t smem = 0;
+  cudaGraphExec_t graph[kServeBuffers] = {};
+};
+}  // namespace mpmi
+
 struct mpmi_server {
   mpmi_ctx* ctx = nullptr;
   const mpmi_model* model = nullptr;
@@ -317,7 +339,6 @@ struct mpmi_server {
   mpmi_result* res_dev[kServeBuffers] = {};
   mpmi_result* res_host[kServeBuffers] = {};         // pinned
   std::vector<int> slots[kServeBuffers];
-  cudaGraphExec_t graph[kServeBuffers] = {};
   cudaStream_t bstream[kServeBuffers] = {};  // each buffer's batches run here
   cudaEvent_t start[kServeBuffers] = {};     // before the graph (timing)
   cudaEvent_t done[kServeBuffers] = {};      // after the graph
@@ -328,9 +349,9 @@ struct mpmi_server {
   cudaStream_t capture = nullptr;
   int stage = 0;  // buffer receiving requests (never in flight)
   int max_in_flight = kServeMaxInFlight;
-  size_t table_bytes = 0, smem = 0;
-  int grid = 0, block = 128;
-  mpmi::ServeKernel kern;
+  size_t table_bytes = 0;
+  mpmi::ServeShape shape;  // the initial or tuned one
+  mpmi::ServeShape large;  // untuned servers: for large batches (no kernel: none)
   uint64_t per_session_bytes = 0, bytes = 0;
 };
 
@@ -345,7 +366,7 @@ static int sfail(cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return sfail(e_, what); \
   } while (0)
 
-static int build_graph(mpmi_server* s, int b) {
+static int build_graph(mpmi_server* s, ServeShape& shape, int b) {
   ServeArgs a;
   memset(&a, 0, sizeof(a));
   a.K = s->model->K32_dev;
@@ -357,12 +378,12 @@ static int build_graph(mpmi_server* s, int b) {
   SRV_CUDA(cudaStreamBeginCapture(s->capture, cudaStreamCaptureModeThreadLocal), "begin capture");
   cudaMemcpyAsync(s->table_dev[b], s->table_host[b], s->table_bytes, cudaMemcpyHostToDevice,
                   s->capture);
-  s->kern.launch(a, s->grid, s->block, s->smem, s->capture);
+  shape.kern.launch(a, shape.grid, shape.block, shape.smem, s->capture);
   cudaMemcpyAsync(s->res_host[b], s->res_dev[b], sizeof(mpmi_result) * s->max_sessions,
                   cudaMemcpyDeviceToHost, s->capture);
   cudaError_t e = cudaStreamEndCapture(s->capture, &g);
   if (e != cudaSuccess) return sfail(e, "end capture");
-  e = cudaGraphInstantiate(&s->graph[b], g, 0);
+  e = cudaGraphInstantiate(&shape.graph[b], g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) return sfail(e, "graph instantiate");
   return MPMI_OK;
@@ -374,26 +395,30 @@ static int build_graph(mpmi_server* s, int b) {
 // taken last are short ones.  Below two tiles per warp the race car loses by a unit's
 // barriers (93k slots 245 -> 274 us), below four the balance bot does (107 us either
 // way).  Mixed sizes and horizons (N log-uniform in 1k..64k, H in 20..100), untuned
-// servers, submit to collect: 24 race cars 850 -> 702 us, 60 2320 -> 1860; 24 balance
-// bots 210 -> 168, 60 455 -> 336; both servers together, 48 sessions 1077 -> 806.  One
-// to six units per block measured the same within 2 % from two on.
-static void plan_batch(mpmi_server* s, ServeHeader* hdr) {
+// servers, one candidate per thread, submit to collect: 24 race cars 850 -> 702 us, 60
+// 2320 -> 1860; 24 balance bots 210 -> 168, 60 455 -> 336; both servers together, 48
+// sessions 1077 -> 806 (713 with large_serve's shape).  One to six units per block measured the same within 2 % from two on.
+// Returns the shape to launch.
+static const ServeShape& plan_batch(const mpmi_server* s, ServeHeader* hdr) {
   SessionTick* ent = reinterpret_cast<SessionTick*>(hdr + 1);
   const int n = hdr->n_requests;
-  const ServeKernel& k = s->kern;
   long long slots = 0;
   for (int i = 0; i < n; ++i) slots += ent[i].n_slots;
+  const ServeShape& shape =
+      s->large.kern.fn != nullptr && slots >= (long long)kLargeBatch * s->ctx->sm_count ? s->large
+                                                                                       : s->shape;
+  const ServeKernel& k = shape.kern;
   std::vector<int> by(n);
   for (int i = 0; i < n; ++i) by[i] = i;
-  const long long warps = (long long)s->grid * (s->block / 32);
+  const long long warps = (long long)shape.grid * (shape.block / 32);
   const int min_tiles = s->model->kind == kCar ? 2 : 4;  // per warp
   hdr->unit = 0;
   if (k.lanes == 1 && slots >= min_tiles * warps * k.per_warp) {
     std::stable_sort(by.begin(), by.end(),
                      [&](int a, int b) { return ent[a].horizon > ent[b].horizon; });
     // a multiple of one tile per warp of a block, about three units per block
-    const int step = k.per_warp * (s->block / 32);
-    const long long want = slots / (3LL * s->grid);
+    const int step = k.per_warp * (shape.block / 32);
+    const long long want = slots / (3LL * shape.grid);
     hdr->unit = (int)std::min<long long>(kServeUnit / step,
                                          std::max<long long>(1, (want + step / 2) / step)) * step;
   }
@@ -408,6 +433,7 @@ static void plan_batch(mpmi_server* s, ServeHeader* hdr) {
   }
   hdr->total = begin;
   hdr->next = 0;
+  return shape;
 }
 
 static int n_flying(const mpmi_server* s) {
@@ -416,9 +442,17 @@ static int n_flying(const mpmi_server* s) {
   return n;
 }
 
+static void drop_graphs(ServeShape& shape) {
+  for (cudaGraphExec_t& g : shape.graph) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  }
+}
+
 static void server_release_device(mpmi_server* s) {
+  drop_graphs(s->shape);
+  drop_graphs(s->large);
   for (int b = 0; b < kServeBuffers; ++b) {
-    if (s->graph[b]) cudaGraphExecDestroy(s->graph[b]);
     for (cudaEvent_t e : {s->start[b], s->done[b], s->after[b]})
       if (e) cudaEventDestroy(e);
     if (s->bstream[b]) cudaStreamDestroy(s->bstream[b]);
@@ -429,6 +463,35 @@ static void server_release_device(mpmi_server* s) {
   }
   cudaFree(s->scratch);
   if (s->capture) cudaStreamDestroy(s->capture);
+}
+
+// Switches a shape record to kernel k with `block` threads per block and a persistent
+// grid (every block resident at once) and captures its batch graphs.  UNSUPPORTED if
+// the shape cannot be resident (the record keeps what it had).
+static int server_set_shape(mpmi_server* s, ServeShape& shape, const ServeKernel& k, int block) {
+  const size_t smem = serve_smem(k, s->model->dev_safety);
+  if (smem > 0 &&
+      cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+          cudaSuccess) {
+    cudaGetLastError();
+    return fail(MPMI_E_UNSUPPORTED, "server: shape cannot take its shared memory");
+  }
+  int nb = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn, block, smem) != cudaSuccess ||
+      nb < 1) {
+    cudaGetLastError();
+    return fail(MPMI_E_UNSUPPORTED, "server: shape cannot be resident");
+  }
+  drop_graphs(shape);
+  shape.kern = k;
+  shape.block = block;
+  shape.smem = smem;
+  shape.grid = nb * s->ctx->sm_count;
+  for (int b = 0; b < kServeBuffers; ++b) {
+    const int rc = build_graph(s, shape, b);
+    if (rc != MPMI_OK) return rc;
+  }
+  return MPMI_OK;
 }
 
 }  // namespace mpmi
@@ -450,12 +513,10 @@ int mpmi_server_create(mpmi_ctx* ctx, const mpmi_model* model, int32_t max_sessi
   s->ctx = ctx;
   s->model = model;
   s->max_sessions = max_sessions;
-  s->kern = kern;
   s->cfg.resize(max_sessions);
   s->used.assign(max_sessions, 0);
   s->state.assign(max_sessions, 0);
   s->table_bytes = sizeof(ServeHeader) + sizeof(SessionTick) * (size_t)max_sessions;
-  s->smem = serve_smem(kern, model->dev_safety);
   s->per_session_bytes =
       sizeof(TickScratch) + kServeBuffers * (sizeof(SessionTick) + sizeof(mpmi_result));
   const uint64_t fixed =
@@ -491,19 +552,18 @@ int mpmi_server_create(mpmi_ctx* ctx, const mpmi_model* model, int32_t max_sessi
     memset(s->table_host[b], 0, s->table_bytes);
     cudaMemset(s->table_dev[b], 0, s->table_bytes);
   }
-  // persistent grid: every block resident at once
-  if (s->smem > 0)
-    cudaFuncSetAttribute(kern.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->smem);
-  int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern.fn, s->block, s->smem);
-  s->grid = (nb < 1 ? 1 : nb) * ctx->sm_count;
-  for (int b = 0; b < kServeBuffers; ++b) {
-    int rc = build_graph(s, b);
-    if (rc != MPMI_OK) {
-      server_release_device(s);
-      delete s;
-      return rc;
+  int rc = server_set_shape(s, s->shape, kern, 128);
+  if (rc == MPMI_OK && large_serve(model->kind).fn != nullptr) {
+    rc = server_set_shape(s, s->large, large_serve(model->kind), 256);
+    if (rc == MPMI_E_UNSUPPORTED) {  // every batch takes the initial shape
+      s->large = ServeShape{};
+      rc = MPMI_OK;
     }
+  }
+  if (rc != MPMI_OK) {
+    server_release_device(s);
+    delete s;
+    return rc;
   }
   s->bytes = fixed;
   ctx->used += fixed;
@@ -631,14 +691,14 @@ int mpmi_server_launch(mpmi_server* s, void* stream, int32_t* n_launched) {
   if (n_flying(s) >= s->max_in_flight)
     return fail(MPMI_E_NOT_READY, "server_launch: the most batches allowed in flight are on the "
                                   "GPU (collect one first)");
-  plan_batch(s, s->table_host[b]);
+  const ServeShape& shape = plan_batch(s, s->table_host[b]);
   // the batch follows the work queued so far on the caller's stream, and runs
   // on its buffer's own stream so that it overlaps the batches in flight
   cudaStream_t st = (cudaStream_t)stream;
   SRV_CUDA(cudaEventRecord(s->after[b], st), "server event");
   SRV_CUDA(cudaStreamWaitEvent(s->bstream[b], s->after[b], 0), "server stream wait");
   SRV_CUDA(cudaEventRecord(s->start[b], s->bstream[b]), "server event");
-  SRV_CUDA(cudaGraphLaunch(s->graph[b], s->bstream[b]), "server graph launch");
+  SRV_CUDA(cudaGraphLaunch(shape.graph[b], s->bstream[b]), "server graph launch");
   SRV_CUDA(cudaEventRecord(s->done[b], s->bstream[b]), "server event");
   if (n_launched) *n_launched = n;
   s->flying[b] = true;
@@ -727,39 +787,6 @@ int mpmi_server_collect(mpmi_server* s, mpmi_result* out, int32_t* slots_out, in
 
 }  // extern "C"
 
-namespace mpmi {
-
-// Switches the server to launch shape k with `block` threads per block and
-// re-captures both batch graphs.  UNSUPPORTED if the shape cannot be resident.
-static int server_set_shape(mpmi_server* s, const ServeKernel& k, int block) {
-  const size_t smem = serve_smem(k, s->model->dev_safety);
-  if (smem > 0 &&
-      cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return fail(MPMI_E_UNSUPPORTED, "server: shape cannot take its shared memory");
-  }
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn, block, smem) != cudaSuccess ||
-      nb < 1) {
-    cudaGetLastError();
-    return fail(MPMI_E_UNSUPPORTED, "server: shape cannot be resident");
-  }
-  s->kern = k;
-  s->block = block;
-  s->smem = smem;
-  s->grid = nb * s->ctx->sm_count;
-  for (int b = 0; b < kServeBuffers; ++b) {
-    if (s->graph[b]) cudaGraphExecDestroy(s->graph[b]);
-    s->graph[b] = nullptr;
-    const int rc = build_graph(s, b);
-    if (rc != MPMI_OK) return rc;
-  }
-  return MPMI_OK;
-}
-
-}  // namespace mpmi
-
 extern "C" {
 
 int mpmi_server_tune(mpmi_server* s, int32_t n, const mpmi_session_config* cfgs,
@@ -787,8 +814,10 @@ int mpmi_server_tune(mpmi_server* s, int32_t n, const mpmi_session_config* cfgs,
   std::vector<int32_t> got(n);
   std::vector<uint64_t> ticks(n);
   std::vector<float> t(reps);
-  const ServeKernel initial = s->kern;
-  const int initial_block = s->block;
+  const ServeKernel initial = s->shape.kern;
+  const int initial_block = s->shape.block;
+  const ServeShape large = s->large;  // every batch takes the shape being timed
+  s->large = ServeShape{};
   ServeKernel best_k = initial;
   int best_block = initial_block;
   mpmi_tune_result best;
@@ -799,7 +828,7 @@ int mpmi_server_tune(mpmi_server* s, int32_t n, const mpmi_session_config* cfgs,
   static const int kBlocks[] = {64, 128, 256};
   for (const ServeKernel& k : serve_shapes(s->model->kind)) {
     for (int block : kBlocks) {
-      rc = server_set_shape(s, k, block);
+      rc = server_set_shape(s, s->shape, k, block);
       if (rc == MPMI_E_UNSUPPORTED) {
         rc = MPMI_OK;
         continue;
@@ -839,8 +868,13 @@ int mpmi_server_tune(mpmi_server* s, int32_t n, const mpmi_session_config* cfgs,
     if (rc != MPMI_OK) break;
   }
   // keep the winner (or go back to the initial shape after a failure)
-  const int rc2 = rc == MPMI_OK ? server_set_shape(s, best_k, best_block)
-                                : server_set_shape(s, initial, initial_block);
+  const int rc2 = server_set_shape(s, s->shape, rc == MPMI_OK ? best_k : initial,
+                                   rc == MPMI_OK ? best_block : initial_block);
+  s->large = large;
+  if (rc == MPMI_OK) {  // a tuned server keeps to its winner
+    drop_graphs(s->large);
+    s->large = ServeShape{};
+  }
   release_all();
   if (rc != MPMI_OK) return rc;
   if (rc2 != MPMI_OK) return rc2;

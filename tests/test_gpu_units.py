@@ -110,3 +110,10 @@ def test_served_units_equal_the_tick_alone(setup, which, sizes):
                 assert got[slots[i]][k] == want[k], (i, k)
             assert np.array_equal(got[slots[i]]["u_r"], want["u_r"])
     srv.free()
+
+
+def test_served_large_batch_equals_the_tick_alone(setup):
+    """A batch past the size at which an untuned race-car server takes two candidates
+    per thread (1,200 slots per SM): ragged ends, one-slot and long-horizon sessions."""
+    sizes = [(131071, 30), (64000, 60), (0, 25), (30011, 100), (33, 20), (65, 40)]
+    test_served_units_equal_the_tick_alone(setup, "car", sizes)
