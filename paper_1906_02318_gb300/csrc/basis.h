@@ -18,6 +18,7 @@
 #pragma once
 
 #include <math.h>
+#include <stdint.h>
 
 #ifdef __CUDACC__
 #define MPMI_HD __host__ __device__ __forceinline__
@@ -129,6 +130,40 @@ MPMI_HD void feature_split(int kind, int j, const T* x, T s, T c, T* a, T* b) {
   } else {
     b[j - nx] = T(1);
   }
+}
+
+// feature_split as data, for code that gives each lane of a warp one feature: with v =
+// {1, x_0 .. x_5, s, c, 0}, a = (v[i] v[j]) v[k] and b_m = v[l], the other b zero; the
+// same products in the same order.  Code: i, j, k, l in nibbles 0..3, m in nibble 4.
+constexpr uint32_t kVOne = 0, kVX = 1, kVSin = 7, kVCos = 8, kVZero = 9;
+constexpr uint32_t code_a(uint32_t i, uint32_t j = kVOne, uint32_t k = kVOne) {
+  return i | j << 4 | k << 8 | kVZero << 12;
+}
+constexpr uint32_t code_b(uint32_t m, uint32_t l) { return kVZero | l << 12 | m << 16; }
+constexpr uint32_t feature_code(int kind, int j) {
+  const uint32_t S = kVSin, C = kVCos;
+  if (kind == kBot) {
+    const uint32_t thd = kVX + 1;
+    const uint32_t f[12] = {code_a(kVX),      code_a(thd),    code_a(kVX + 2),
+                            code_a(kVX + 3),  code_b(0, kVOne), code_a(S),
+                            code_a(C),        code_a(thd, thd), code_b(0, thd),
+                            code_a(thd, thd, S), code_b(0, C),  code_a(kVOne)};
+    return f[j];
+  }
+  if (kind == kCar) {
+    const uint32_t vx = kVX + 3, vy = kVX + 4, om = kVX + 5;
+    const uint32_t f[32] = {
+        code_a(kVX),      code_a(kVX + 1),  code_a(kVX + 2),  code_a(vx),       code_a(vy),
+        code_a(om),       code_b(0, kVOne), code_b(1, kVOne), code_a(S),        code_a(C),
+        code_a(vx, C),    code_a(vx, S),    code_a(vy, C),    code_a(vy, S),    code_a(om, vx),
+        code_a(om, vy),   code_a(vx, vx),   code_a(vy, vy),   code_a(om, om),   code_b(0, vx),
+        code_b(0, vy),    code_b(0, om),    code_b(1, vx),    code_b(0, C),     code_b(0, S),
+        code_b(1, C),     code_b(1, S),     code_a(om, C),    code_a(om, S),    code_a(vx, vy),
+        code_b(2, kVOne), code_a(kVOne)};
+    return f[j];
+  }
+  const int nx = kind == kLin11 ? 1 : kind == kLin22 ? 2 : 4;
+  return j < nx ? code_a(kVX + j) : code_b(j - nx, kVOne);
 }
 
 // Features that depend on the input alone (and the constant).  With the input

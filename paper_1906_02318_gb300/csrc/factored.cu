@@ -104,16 +104,29 @@ __device__ __forceinline__ int first_violation(const DevTrack& tr, const TrackVi
   return bad != 0u ? __ffs(bad) - 1 : 32;
 }
 
+// The lifting's feature codes of a basis.
+struct FeatureCodes {
+  uint32_t c[32];
+};
+constexpr FeatureCodes feature_codes(int kind, int n) {
+  FeatureCodes f{};
+  for (int j = 0; j < n; ++j) f.c[j] = feature_code(kind, j);
+  return f;
+}
+template <int KIND>
+__device__ const FeatureCodes g_codes = feature_codes(KIND, BasisTraits<KIND>::N);
+
 // One tick in the factorised form.  Dynamic shared memory: [track grid (race
 // car)] [V: H x ro_n float4, (a, b_1, b_2, b_3) coefficients per read-out].
 // One block per SM.  A block draws up to a thread's candidate each, then its warps take
 // the drawn candidates from a counter and test 32 steps of one at a time (the read-outs
 // of different steps do not depend on each other; lane l: step t0 + l + 1), until the
 // first violation.  Bound: issue, about 190 instructions per 32 steps, the track test
-// most of them.  GB300, race car, N = 30001, H = 100: 25.6 us; 56.7 with 760 blocks of
+// most of them.  GB300, race car, N = 30001, H = 100: 19.8 us; 56.7 with 760 blocks of
 // 128 threads that each staged the grid and built V, gave some warps two tiles and
 // others one, and tested every listed segment of every step; 28.0 with equal tiles per
-// warp and one feature per lane in the prologue (10k cycles of a 32-way switch).
+// warp; 25.6 with the lifting's features in code (a 32-way switch, or one after the
+// other by a whole warp: 11k cycles) instead of one per lane from their codes (300).
 template <int KIND>
 __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_constant__ TickArgs a) {
   using B = BasisTraits<KIND>;
@@ -178,25 +191,30 @@ __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_const
 #pragma unroll
     for (int j = 0; j < N4; ++j) p4[j] = __ldg(row + j);
   }
+  const uint32_t code = warp == 0 && lane < N ? g_codes<KIND>.c[lane] : 0u;
   if (sure) grid_dep_wait();
 
   float uh[NU];
 #pragma unroll
   for (int j = 0; j < NU; ++j) uh[j] = __double2float_rn(a.u_h[j]);
   if (warp == 0) {
-    // every feature in straight-line code by each lane of one warp (one feature per
-    // lane would take the switch's 32 ways one after the other)
-    float xs[NX], sn = 0.f, cs = 1.f;
-#pragma unroll
-    for (int j = 0; j < NX; ++j) xs[j] = __double2float_rn(a.x_t[j]);
-    if constexpr (ANG >= 0) sincosf(xs[ANG], &sn, &cs);
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-      float av, bv[kMaxP];
-      feature_split<float>(KIND, j, xs, sn, cs, &av, bv);
-      if (lane == (j & 31))
-        s_f[j] = make_float4(av, bv[0], NP > 1 ? bv[1] : 0.f, NP > 2 ? bv[2] : 0.f);
+    // one feature per lane; lane i holds v[i] of the feature codes
+    float v = 0.f;
+    if (lane >= (int)kVX && lane < (int)kVX + NX) v = __double2float_rn(a.x_t[lane - kVX]);
+    if (lane == (int)kVOne) v = 1.f;
+    if constexpr (ANG >= 0) {
+      float sn, cs;
+      sincosf(__shfl_sync(kFull, v, kVX + ANG), &sn, &cs);
+      if (lane == (int)kVSin) v = sn;
+      if (lane == (int)kVCos) v = cs;
     }
+    const float f0 = __shfl_sync(kFull, v, code & 15), f1 = __shfl_sync(kFull, v, code >> 4 & 15);
+    const float f2 = __shfl_sync(kFull, v, code >> 8 & 15);
+    const float b = __shfl_sync(kFull, v, code >> 12 & 15);
+    const uint32_t m = code >> 16;
+    if (lane < N)
+      s_f[lane] = make_float4(__fmul_rn(__fmul_rn(f0, f1), f2), m == 0 ? b : 0.f,
+                              m == 1 ? b : 0.f, m == 2 ? b : 0.f);
   }
   __syncthreads();
   // V[t][r] = (P_t row ro_idx[r]) . (a, b_1, b_2, b_3)
