@@ -122,7 +122,7 @@ __device__ const FeatureCodes g_codes = feature_codes(KIND, BasisTraits<KIND>::N
 // the drawn candidates from a counter and test 32 steps of one at a time (the read-outs
 // of different steps do not depend on each other; lane l: step t0 + l + 1), until the
 // first violation.  Bound: issue, about 190 instructions per 32 steps, the track test
-// most of them.  GB300, race car, N = 30001, H = 100: 19.8 us; 56.7 with 760 blocks of
+// most of them.  GB300, race car, N = 30001, H = 100: 20.2 us; 56.7 with 760 blocks of
 // 128 threads that each staged the grid and built V, gave some warps two tiles and
 // others one, and tested every listed segment of every step; 28.0 with equal tiles per
 // warp; 25.6 with the lifting's features in code (a 32-way switch, or one after the
@@ -264,14 +264,17 @@ __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_const
 
   unsigned long long best = ~0ull;
   unsigned int n_safe = 0, n_exec = 0;
-  const int first = (int)blockIdx.x * share;
-  const int end = failed ? first : min(first + share, n_eval);
-  for (int base = first; base < end; base += (int)blockDim.x) {
-    const int cnt = min((int)blockDim.x, end - base);
+  // the block's candidates, in chunks dealt out in turn (a grid's or a caller's samples
+  // may come in order, and long-lived ones would meet in a few blocks)
+  const UnitSlots in{(int)blockIdx.x, n_active};
+  const int mine = failed ? 0 : unit_count(n_eval, n_active, (int)blockIdx.x);
+  for (int base = 0; base < mine; base += (int)blockDim.x) {
+    const int cnt = min((int)blockDim.x, mine - base);
     int slot = 0;
     float cost = 0.f;
     if (tid < cnt) {
-      slot = a.slot_list ? a.slot_list[base + tid] : base + tid;
+      slot = in.slot(base + tid);
+      if (a.slot_list) slot = a.slot_list[slot];
       float xi[NU], p[NP];
       candidate_value<NU>(a, slot, uh, xi);
 #pragma unroll

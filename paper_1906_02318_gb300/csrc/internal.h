@@ -55,7 +55,7 @@ struct TickArgs {
   const float* ext;    // device samples N x nu (EXTERNAL) or null
   DevSafety safety;
   int kind;            // BasisKind
-  int unit;            // slots a block sorts and runs at a time (0: unsorted tiles)
+  int unit, n_units;   // most slots of a sorted unit (0: unsorted tiles), number of units
   int n_samples, n_slots, horizon, include_user, sampler;
   float in_lo[MPMI_MAX_NU], in_w[MPMI_MAX_NU];        // float32 box (UNIFORM)
   double in_lo64[MPMI_MAX_NU], in_hi64[MPMI_MAX_NU];  // float64 box (GRID)
@@ -164,7 +164,7 @@ struct mpmi_session {
   // the few-candidate shape)
   int max_grid[16] = {};
   size_t grid_smem[16] = {};
-  int unit[16] = {};               // the launch kind's sorted units (one-lane shapes)
+  int n_units[16] = {};            // the launch kind's sorted units (0: unsorted tiles)
   mpmi::TickScratch* scratch_dev = nullptr;
   mpmi_result* result_dev = nullptr;
   double* in_dev = nullptr;        // x_t (8 doubles) then u_h (4 doubles)

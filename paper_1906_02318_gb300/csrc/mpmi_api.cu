@@ -336,8 +336,11 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
   const int n_work = (n_hint > 0 && n_hint < s->n_slots) ? n_hint : s->n_slots;
   if (s->max_grid[t] == 0 || s->grid_smem[t] != smem) {
     int nb = 0;
-    s->unit[t] = 0;
-    if (k.fn_units && a.slot_list == nullptr) {
+    s->n_units[t] = 0;
+    // a grid over one input comes in order as it is (N = 522070, H = 80: 97 us, 109 sorted
+    // again)
+    const bool ordered = a.sampler == MPMI_SAMPLER_GRID && s->model->nu == 1;
+    if (k.fn_units && a.slot_list == nullptr && !ordered) {
       const size_t most = smem + unit_bytes(kUnitMax);
       cudaError_t e =
           cudaFuncSetAttribute(k.fn_units, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -349,10 +352,10 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
       if (nb > 0 && units_pay(s->model->kind, n_work, blocks * (block / 32) * per_warp)) {
         // equal shares of the slots per block, in as few rounds as kUnitMax allows
         const long long rounds = (n_work + blocks * kUnitMax - 1) / (blocks * kUnitMax);
-        s->unit[t] = (int)((n_work + blocks * rounds - 1) / (blocks * rounds));
+        s->n_units[t] = (int)(blocks * rounds);
       }
     }
-    if (s->unit[t] == 0) {
+    if (s->n_units[t] == 0) {
       // static (lane exchange) plus dynamic shared memory may pass the 48 KB default
       if (smem > 0) {
         cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -366,9 +369,14 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
     s->max_grid[t] = nb * s->ctx->sm_count;
     s->grid_smem[t] = smem;
   }
-  a.unit = s->unit[t];
-  const int per_block = a.unit > 0 ? a.unit : per_warp * (block / 32);
+  const int per_block = per_warp * (block / 32);
   int grid = (n_work + per_block - 1) / per_block;
+  a.n_units = s->n_units[t];
+  a.unit = 0;
+  if (a.n_units > 0) {
+    a.unit = unit_count(n_work, a.n_units, 0);  // no unit has more slots than the first
+    grid = a.n_units;
+  }
   if (grid > s->max_grid[t]) grid = s->max_grid[t];
   if (a.unit > 0) k.launch_units(a, grid, block, smem + unit_bytes(a.unit), st);
   else k.launch(a, grid, block, smem, st);

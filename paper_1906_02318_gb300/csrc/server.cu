@@ -206,12 +206,14 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
       const int base = (u - ent[r].range_begin) * unit;
       const int cnt = min(unit, st.n_slots - base);
       load_state(st, req);
-      const uint16_t* order = sort_unit<NU>(st, dyn_of(st), base, cnt, unit, uh, buf, &s_tile);
+      const UnitSlots in{base / kUnitChunk, 1};  // a unit is whole tiles, 32 slots at least
+      const uint16_t* order = sort_unit<NU>(st, dyn_of(st), in, cnt, unit, uh, buf, &s_tile);
       __syncthreads();
       if (tid == 0) {
         s_unit = atomicAdd(&hdr->next, 1);  // read after the unit's last barrier
         s_best = ~0ull;
         s_cnt = 0ull;
+        s_tile = 0;
       }
       __syncthreads();
       unsigned long long best = ~0ull;
@@ -223,7 +225,7 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
         if (wt * PER_WARP >= cnt) break;
         run_tile<KIND, L, C, KSMEM, false, false, true, false>(
             st, dyn_of(st), sa.safety, wt, cnt, xs, uh, sn, cs, kr, sK4, tv,
-            &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec, order, base);
+            &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec, order, in);
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {

@@ -701,6 +701,23 @@ __device__ __forceinline__ void fma_word(const float4 kv, const float* z, int w,
   v = __fmaf_rn(kv.w, z[staged_col(KIND, N, 4 * w + 3)], v);
 }
 
+// The slots of a sorted unit (see sort_unit): chunks of kUnitChunk consecutive slots,
+// `stride` chunks apart, the first one number `first`.
+constexpr int kUnitChunk = 8;
+struct UnitSlots {
+  int first, stride;
+  __device__ __forceinline__ int slot(int i) const {
+    return (i / kUnitChunk * stride + first) * kUnitChunk + i % kUnitChunk;
+  }
+};
+// Unit u of n_units over n slots: chunks u, u + n_units, ...; its number of slots.
+MPMI_HD int unit_count(int n, int n_units, int u) {
+  const int chunks = (n + kUnitChunk - 1) / kUnitChunk;
+  if (u >= chunks) return 0;
+  const int mine = (chunks - u + n_units - 1) / n_units;
+  return mine * kUnitChunk - ((chunks - 1) % n_units == u ? chunks * kUnitChunk - n : 0);
+}
+
 // One warp-tile: the PER_WARP = 32 C / L candidate positions wt * PER_WARP ...
 // of a tick (Alg. 2 for each: sample, lift, predict with early exit, test,
 // score), folded into the caller's running key minimum and counts.  P is the
@@ -723,7 +740,7 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
                                          const KR& kr, const float4* sK4, const TrackView& tv,
                                          float* xbuf, unsigned long long& best,
                                          unsigned int& n_safe, unsigned int& n_exec,
-                                         const uint16_t* order = nullptr, int base = 0) {
+                                         const uint16_t* order = nullptr, UnitSlots in = {0, 1}) {
   using B = BasisTraits<KIND>;
   constexpr int N = B::N, NX = B::NX, NU = B::NU, NP = B::NP;
   constexpr int R = N / L;
@@ -749,8 +766,8 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
     valid[c] = pos < n_eval;
     if constexpr (L == 1) {
       // a tile of a sorted unit (sort_unit): position pos of the unit is slot
-      // base + order[pos]
-      if (order != nullptr && valid[c]) pos = base + (int)order[pos];
+      // in.slot(order[pos])
+      if (order != nullptr && valid[c]) pos = in.slot((int)order[pos]);
     }
     slot[c] = (valid[c] && a.slot_list) ? a.slot_list[pos] : pos;
     float xi[NU];
@@ -1187,10 +1204,15 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
 // a unit by the first input (a counting sort over kUnitBins bins of the input box)
 // and lets its warps take the unit's tiles from a counter: a tile's candidates then
 // leave together, and warps that the scheduler favours take more tiles.  The order
-// changes no result (a minimum, integer sums, per-slot outputs).
-// GB300, ticks back to back: balance bot H = 50, N = 1048576 207 -> 164 us, H = 100,
-// N = 200000 86 -> 44 us; race car H = 60, N = 65536 150 -> 145 us, N = 262144 578 ->
-// 460 us, H = 100, N = 131072 518 -> 322 us.
+// changes no result (a minimum, integer sums, per-slot outputs).  A unit's slots are
+// chunks from all over the tick: a caller's samples, or a grid's, may come in order, and
+// with a run of them per block the long-lived ones met in a few blocks (balance bot,
+// grid, N = 522070, H = 80: 189 us, 109 in chunks).  A grid over one input needs no
+// sorting at all and takes unsorted tiles (97 us; launch_tick_args).
+// GB300, ticks back to back: balance bot H = 50, N = 1048576 207 -> 162 us, H = 100,
+// N = 200000 86 -> 44 us; race car H = 60, N = 65536 150 -> 142 us, N = 262144 578 ->
+// 460 us, H = 100, N = 131072 518 -> 322 us.  Samples already in order of the first
+// input lose what the sorting costs (balance bot, N = 522070, H = 80: 87 -> 92 us).
 constexpr int kUnitMax = 8192, kUnitBins = 256;
 
 // Shared-memory bytes of a unit: bin counters, each candidate's place and bin.
@@ -1198,10 +1220,11 @@ MPMI_HD constexpr size_t unit_bytes(int unit) {
   return 4 * kUnitBins + (3 * (size_t)unit + 15) / 16 * 16;
 }
 
-// Orders positions 0 .. cnt - 1 (slots base + position) by bins of the first input and
-// restarts the tile counter (whole block; buf: unit_bytes(unit) of shared memory).
+// Orders positions 0 .. cnt - 1 (slots in.slot(position)) by bins of the first input and
+// restarts the tile counter behind the warps' first tiles (whole block; buf:
+// unit_bytes(unit) of shared memory).
 template <int NU, class P>
-__device__ __forceinline__ const uint16_t* sort_unit(const P& a, TickDyn d, int base, int cnt,
+__device__ __forceinline__ const uint16_t* sort_unit(const P& a, TickDyn d, UnitSlots in, int cnt,
                                                      int unit, const float* uh, char* buf,
                                                      int* next) {
   uint32_t* bins = reinterpret_cast<uint32_t*>(buf);
@@ -1210,12 +1233,12 @@ __device__ __forceinline__ const uint16_t* sort_unit(const P& a, TickDyn d, int 
   const int tid = threadIdx.x;
   const float scale = (float)kUnitBins / a.in_w[0];
   __syncthreads();  // every warp is done with the previous unit
-  if (tid == 0) *next = 0;
+  if (tid == 0) *next = blockDim.x >> 5;  // the warps' first tiles
   for (int b = tid; b < kUnitBins; b += blockDim.x) bins[b] = 0;
   __syncthreads();
   for (int i = tid; i < cnt; i += blockDim.x) {
     float xi[NU];
-    candidate_value<NU>(a, d.t_lo, d.t_hi, base + i, uh, xi);
+    candidate_value<NU>(a, d.t_lo, d.t_hi, in.slot(i), uh, xi);
     // out-of-box and NaN inputs land in an end bin
     const float f = fminf(fmaxf((xi[0] - a.in_lo[0]) * scale, 0.f), (float)(kUnitBins - 1));
     bin[i] = (uint8_t)f;
@@ -1471,31 +1494,30 @@ __global__ void __launch_bounds__(kMaxBlock) tick_kernel(const __grid_constant__
   unsigned int n_safe = 0, n_exec = 0;
   const int wpb = blockDim.x >> 5;
   constexpr int PER_WARP = GPW * C;  // candidate slots per warp-tile
-  const auto tile = [&](int wt, int cnt, const uint16_t* order, int base) {
+  const auto tile = [&](int wt, int cnt, const uint16_t* order, UnitSlots in) {
     // sorted tiles of two candidates per thread keep the pipes full without piping
     run_tile<KIND, L, C, KSMEM, TRAJ, NOISE, !PARTIALS, !(UNITS && C == 2)>(
         a, dyn_of(a), a.safety, wt, cnt, xs, uh, sn, cs, kr, sK4, tv,
-        &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec, order, base);
+        &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec, order, in);
   };
   if constexpr (UNITS) {
     char* buf = reinterpret_cast<char*>(s_dyn + KWORDS) +
                 (track_on ? a.safety.track.blob_bytes : 0);
-    for (int base = failed ? n_eval : (int)blockIdx.x * a.unit; base < n_eval;
-         base += (int)gridDim.x * a.unit) {
-      const int cnt = min(a.unit, n_eval - base);
-      const uint16_t* order = sort_unit<NU>(a, dyn_of(a), base, cnt, a.unit, uh, buf, &s_next);
-      while (true) {
-        int wt = 0;
-        if (lane == 0) wt = atomicAdd(&s_next, 1);
-        wt = __shfl_sync(kFull, wt, 0);
-        if (wt * PER_WARP >= cnt) break;
-        tile(wt, cnt, order, base);
+    for (int u = failed ? a.n_units : (int)blockIdx.x; u < a.n_units; u += (int)gridDim.x) {
+      const UnitSlots in{u, a.n_units};
+      const int cnt = unit_count(n_eval, a.n_units, u);
+      const uint16_t* order = sort_unit<NU>(a, dyn_of(a), in, cnt, a.unit, uh, buf, &s_next);
+      for (int wt = warp; wt * PER_WARP < cnt;) {
+        tile(wt, cnt, order, in);
+        int next = 0;
+        if (lane == 0) next = atomicAdd(&s_next, 1);
+        wt = __shfl_sync(kFull, next, 0);
       }
     }
   } else {
     const int n_wtiles = failed ? 0 : (n_eval + PER_WARP - 1) / PER_WARP;
     for (int wt = blockIdx.x * wpb + warp; wt < n_wtiles; wt += gridDim.x * wpb)
-      tile(wt, n_eval, nullptr, 0);
+      tile(wt, n_eval, nullptr, UnitSlots{0, 1});
   }
   // the next launch may start once every block is here: its start overlaps the
   // reduction, and no block of it takes an SM's place from a tick that still runs
