@@ -92,7 +92,7 @@ __device__ __forceinline__ int first_violation(const DevTrack& tr, const TrackVi
     unsigned int todo = __ballot_sync(kFull, cell.open), taken;
     if (bad != 0u) todo &= (bad & (0u - bad)) - 1u;  // before the first violation
     while (todo != 0u) {
-      const unsigned int got = settle_open(tr, tv, px, py, cell, todo, &taken);
+      const unsigned int got = settle_open<1>(tr, tv, px, py, cell, todo, &taken);
       if ((taken & ~got) != 0u) {  // an earlier violation than any left open
         bad |= taken & ~got;
         break;
@@ -122,7 +122,7 @@ __device__ const FeatureCodes g_codes = feature_codes(KIND, BasisTraits<KIND>::N
 // the drawn candidates from a counter and test 32 steps of one at a time (the read-outs
 // of different steps do not depend on each other; lane l: step t0 + l + 1), until the
 // first violation.  Bound: issue, about 190 instructions per 32 steps, the track test
-// most of them.  GB300, race car, N = 30001, H = 100: 20.2 us; 56.7 with 760 blocks of
+// most of them.  GB300, race car, N = 30001, H = 100: 19.6 us; 56.7 with 760 blocks of
 // 128 threads that each staged the grid and built V, gave some warps two tiles and
 // others one, and tested every listed segment of every step; 28.0 with equal tiles per
 // warp; 25.6 with the lifting's features in code (a 32-way switch, or one after the

@@ -461,15 +461,18 @@ __device__ __forceinline__ bool seg_hit(const DevTrack& tr, const TrackView& v, 
 }
 
 // isSafe on the track part with one position per lane, in two stages.  A lane in a
-// boundary cell tests the first two listed segments (nearest to the cell first), which
-// settles most positions on the road (track_cell).  The warp then settles the open
+// boundary cell tests the first listed segment (nearest to the cell first), which settles
+// the positions on the road but 1 in 300 (track_cell; a second one settles 3 in 1000 and
+// costs every lane the test).  The warp then settles the open
 // ones together, four at a time: eight lanes test eight listed segments of one
 // position per round (settle_open).  A lane that tests its whole list alone (7 to 15
 // entries when the position is off the road) keeps the other 31 waiting through every
 // round.  Race car, one lane per candidate: N = 16384 69 -> 64 us, N = 32768 95 -> 91
-// us, the tensor-core rollout at N = 65536 79.7 -> 78.4 us.
+// us, the tensor-core rollout at N = 65536 79.7 -> 78.4 us; one segment instead of two
+// in the first stage: 77.1 -> 76.0 us there, factorised N = 30001 20.2 -> 19.6, two
+// candidates per thread N = 65536 142.5 -> 141.5.
 struct TrackCell {
-  bool ok, open;  // on the road; undecided after the first two segments
+  bool ok, open;  // on the road; undecided after the first stage
   int off, cnt;   // the cell's list
 };
 
@@ -486,11 +489,8 @@ __device__ __forceinline__ TrackCell track_cell(const DevTrack& tr, const TrackV
       if (cls == kCellBoundary) {
         r.off = (int)((c >> 2) & 0x3FFFFFu);
         r.cnt = (int)(c >> 24);
-        // entries past the list's end repeat its last one (a list is never empty)
-        const bool h0 = seg_hit(tr, v, v.list[r.off], px, py);
-        const bool h1 = seg_hit(tr, v, v.list[r.off + min(1, r.cnt - 1)], px, py);
-        r.ok = h0 | h1;
-        r.open = !r.ok & (r.cnt > 2);
+        r.ok = seg_hit(tr, v, v.list[r.off], px, py);  // a list is never empty
+        r.open = !r.ok & (r.cnt > 1);
       }
     }
   }
@@ -498,9 +498,11 @@ __device__ __forceinline__ TrackCell track_cell(const DevTrack& tr, const TrackV
 }
 
 // Takes up to four lanes off `todo` (not 0; lowest first), tests their positions and
-// returns the lanes on the road; *taken: the lanes tested.  All 32 lanes of a warp
+// returns the lanes on the road; *taken: the lanes tested.  FIRST: the listed segments
+// that the first stage has tested.  All 32 lanes of a warp
 // call it together (it shuffles over the full warp): never under a branch that some
 // lanes skip.
+template <int FIRST>
 __device__ __forceinline__ unsigned int settle_open(const DevTrack& tr, const TrackView& v,
                                                     float px, float py, const TrackCell& cell,
                                                     unsigned int& todo, unsigned int* taken) {
@@ -521,7 +523,7 @@ __device__ __forceinline__ unsigned int settle_open(const DevTrack& tr, const Tr
   const float qx = __shfl_sync(kFull, px, mine), qy = __shfl_sync(kFull, py, mine);
   const int qo = __shfl_sync(kFull, cell.off, mine), qc = __shfl_sync(kFull, cell.cnt, mine);
   bool hit = false;
-  for (int i = 2 + (lane & 7); i < qc && !hit; i += 16) {
+  for (int i = FIRST + (lane & 7); i < qc && !hit; i += 16) {
     const bool h0 = seg_hit(tr, v, v.list[qo + i], qx, qy);
     const bool h1 = seg_hit(tr, v, v.list[qo + min(i + 8, qc - 1)], qx, qy);
     hit = h0 | h1;
@@ -531,8 +533,8 @@ __device__ __forceinline__ unsigned int settle_open(const DevTrack& tr, const Tr
 }
 
 // The first stage without branches, for code that runs it beside other work; an
-// inactive lane reads entry 0 of the lists.  L = 2: the two lanes of a candidate test
-// one of the first two segments each; L >= 8: a candidate's lanes test the first
+// inactive lane reads entry 0 of the lists.  L = 1: the first segment; L = 2: the two
+// lanes of a candidate test one of the first two each; L >= 8: a candidate's lanes test the first
 // sixteen segments (track_settle joins them).
 template <int L>
 __device__ __forceinline__ TrackCell track_front(const DevTrack& tr, const TrackView& v, float px,
@@ -547,7 +549,7 @@ __device__ __forceinline__ TrackCell track_front(const DevTrack& tr, const Track
   TrackCell r;
   r.off = edge ? (int)((c >> 2) & 0x3FFFFFu) : 0;
   r.cnt = edge ? (int)(c >> 24) : 1;
-  constexpr int FIRST = L <= 2 ? 2 : 16;  // segments the candidate's lanes test here
+  constexpr int FIRST = L <= 2 ? L : 16;  // segments the candidate's lanes test here
   bool hit = false;
 #pragma unroll
   for (int i = 0; i < FIRST / L; ++i)
@@ -583,7 +585,7 @@ __device__ __forceinline__ bool track_settle(const DevTrack& tr, const TrackView
     todo &= (todo >> 1) & 0x55555555u;
   }
   while (todo != 0u) {
-    const unsigned int got = settle_open(tr, v, px, py, cell, todo, &taken);
+    const unsigned int got = settle_open<L>(tr, v, px, py, cell, todo, &taken);
     ok |= L == 2 ? got | (got << 1) : got;
   }
   return ((ok >> (threadIdx.x & 31)) & 1u) != 0u;
@@ -595,7 +597,7 @@ __device__ __forceinline__ bool track_ok_warp(const DevTrack& tr, const TrackVie
                                               float py, bool active) {
   TrackCell cell = track_cell(tr, v, px, py, active);
   unsigned int todo = __ballot_sync(kFull, cell.open), got = 0u, taken;
-  while (todo != 0u) got |= settle_open(tr, v, px, py, cell, todo, &taken);
+  while (todo != 0u) got |= settle_open<1>(tr, v, px, py, cell, todo, &taken);
   return cell.ok | (((got >> (threadIdx.x & 31)) & 1u) != 0u);
 }
 
