@@ -534,32 +534,40 @@ __device__ __forceinline__ unsigned int settle_open(const DevTrack& tr, const Tr
 
 // The first stage without branches, for code that runs it beside other work; an
 // inactive lane reads entry 0 of the lists.  L = 1: the first segment; L = 2: the two
-// lanes of a candidate test one of the first two each; L >= 8: a candidate's lanes test the first
-// sixteen segments (track_settle joins them).
-template <int L>
-__device__ __forceinline__ TrackCell track_front(const DevTrack& tr, const TrackView& v, float px,
-                                                 float py, bool active, int q) {
+// lanes of a candidate test one of the first two each; L >= 8: a candidate's lanes test
+// the first sixteen segments (track_settle joins them).  Two halves, each one table
+// read deep: track_look reads the cell (ok: inside one; open: in a boundary cell), track_near tests
+// the segments.
+__device__ __forceinline__ TrackCell track_look(const DevTrack& tr, const TrackView& v, float px,
+                                                float py, bool active) {
   const float fx = (px - tr.gx0) * tr.inv_h;
   const float fy = (py - tr.gy0) * tr.inv_h;
   const bool in = active & (fx >= 0.f) & (fx < (float)tr.gnx) & (fy >= 0.f) & (fy < (float)tr.gny);
   const int ix = (int)fx, iy = (int)fy;
   const uint32_t c = v.cells[in ? iy * tr.gnx + ix : 0];
   const uint32_t cls = in ? c & 3u : (uint32_t)kCellOutside;
-  const bool edge = cls == kCellBoundary;
   TrackCell r;
-  r.off = edge ? (int)((c >> 2) & 0x3FFFFFu) : 0;
-  r.cnt = edge ? (int)(c >> 24) : 1;
+  r.ok = cls == kCellInside;
+  r.open = cls == kCellBoundary;
+  r.off = r.open ? (int)((c >> 2) & 0x3FFFFFu) : 0;
+  r.cnt = r.open ? (int)(c >> 24) : 1;
+  return r;
+}
+
+template <int L>
+__device__ __forceinline__ TrackCell track_near(const DevTrack& tr, const TrackView& v, float px,
+                                                float py, TrackCell r, int q) {
   constexpr int FIRST = L <= 2 ? L : 16;  // segments the candidate's lanes test here
   bool hit = false;
 #pragma unroll
   for (int i = 0; i < FIRST / L; ++i)
     hit = hit | seg_hit(tr, v, v.list[r.off + min(q + i * L, r.cnt - 1)], px, py);
-  r.ok = (cls == kCellInside) | (edge & hit);
-  r.open = edge & !hit & (r.cnt > FIRST);
+  r.ok = r.ok | (r.open & hit);
+  r.open = r.open & !hit & (r.cnt > FIRST);
   return r;
 }
 
-// The second stage for track_front's answer, by whole warps.
+// The second stage for track_near's answer, by whole warps.
 template <int L>
 __device__ __forceinline__ bool track_settle(const DevTrack& tr, const TrackView& v, float px,
                                              float py, const TrackCell& cell, int q) {
@@ -1120,26 +1128,51 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
   // (N = 16384, two lanes) 57.0 -> 53.3.  Served batches and sorted tiles of two
   // candidates per thread keep the pipes full without it (3 and 1 % slower piped).
   constexpr bool PIPE = PIPED && B::TRACK && HELD && (KSMEM ? L <= 2 : L >= 8);
+  // Two steps deep with eight or more lanes (one warp per sub-partition, so a step's
+  // latency counts): the cell is read beside one product, the segments are tested
+  // beside the next, for a second step computed for nothing.  H = 60, sixteen lanes (N =
+  // 1024) 20.5 -> 17.8 us, eight (N = 2400) 24.0 -> 22.4, eight and two warps (N = 4096)
+  // 28.2 -> 26.7; two lanes lose (N = 16384 50.9 -> 54.0).  Trajectories keep one step.
+  constexpr bool DEEP = PIPE && !TRAJ && L >= 8;
   if (PIPE && safety.has_track) {
     if constexpr (PIPE) {
-      advance(1);
-      for (int t = 1; t <= H; ++t) {
-        perturb(t);
-        record(t);
-        TrackCell cell[C];
-        float px[C], py[C];
+      TrackCell look[C];
+      float px[C], py[C];
+      const auto look_at = [&](TrackCell* cell, float* x, float* y) {
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-          px[c] = z[c][0];
-          py[c] = z[c][1];
-          cell[c] = track_front<L>(safety.track, tv, px[c], py[c],
-                                   alive[c] & box_ok<NX>(safety, z[c]), q);
+          x[c] = z[c][0];
+          y[c] = z[c][1];
+          cell[c] = track_look(safety.track, tv, x[c], y[c], alive[c] & box_ok<NX>(safety, z[c]));
         }
-        advance(t + 1);
+      };
+      advance(1);
+      if constexpr (DEEP) {
+        perturb(1);
+        look_at(look, px, py);
+        advance(2);
+      }
+      for (int t = 1; t <= H; ++t) {
+        TrackCell cell[C];
+        float x[C], y[C];
+        if constexpr (DEEP) {
+          perturb(t + 1);
+#pragma unroll
+          for (int c = 0; c < C; ++c) cell[c] = look[c], x[c] = px[c], y[c] = py[c];
+          look_at(look, px, py);
+        } else {
+          perturb(t);
+          record(t);
+          look_at(cell, x, y);
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+          cell[c] = track_near<L>(safety.track, tv, x[c], y[c], cell[c], q);
+        advance(DEEP ? t + 2 : t + 1);
         bool any_alive = false;
 #pragma unroll
         for (int c = 0; c < C; ++c) {
-          const bool ok = track_settle<L>(safety.track, tv, px[c], py[c], cell[c], q);
+          const bool ok = track_settle<L>(safety.track, tv, x[c], y[c], cell[c], q);
           if (alive[c]) {
             if (ok) ttv[c] = t;
             else alive[c] = false;
