@@ -227,13 +227,13 @@ struct DeviceGuard {
 };
 
 #ifdef __CUDACC__
-// Launches a kernel as a programmatic dependent of the one before it on the stream: it
-// may start while that one still runs, and calls grid_dep_wait before it touches
+// Launches a kernel, if `early` as a programmatic dependent of the one before it on the
+// stream: it may start while that one still runs, and calls grid_dep_wait before it touches
 // anything another kernel may write.  (After a kernel that never calls
 // grid_dep_release, or after a copy, it starts when that has ended.)
 template <class... KA, class... A>
-static cudaError_t launch_dependent(void (*fn)(KA...), int grid, int block, size_t smem,
-                                    cudaStream_t st, A&&... args) {
+static cudaError_t launch_early(bool early, void (*fn)(KA...), int grid, int block, size_t smem,
+                                cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3((unsigned)block);
@@ -243,8 +243,13 @@ static cudaError_t launch_dependent(void (*fn)(KA...), int grid, int block, size
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = early ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, fn, std::forward<A>(args)...);
+}
+template <class... KA, class... A>
+static cudaError_t launch_dependent(void (*fn)(KA...), int grid, int block, size_t smem,
+                                    cudaStream_t st, A&&... args) {
+  return launch_early(true, fn, grid, block, smem, st, std::forward<A>(args)...);
 }
 #endif
 

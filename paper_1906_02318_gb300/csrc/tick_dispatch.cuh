@@ -13,17 +13,18 @@ namespace mpmi {
 
 struct TickKernel {
   const void* fn = nullptr;
-  void (*launch)(const TickArgs&, int, int, size_t, cudaStream_t) = nullptr;
+  void (*launch)(const TickArgs&, int, int, size_t, cudaStream_t, bool early) = nullptr;
   size_t k_smem = 0;  // bytes of K staged in shared memory
   // the same shape over sorted units (one lane, no trajectories)
   const void* fn_units = nullptr;
-  void (*launch_units)(const TickArgs&, int, int, size_t, cudaStream_t) = nullptr;
+  void (*launch_units)(const TickArgs&, int, int, size_t, cudaStream_t, bool early) = nullptr;
 };
 
 template <int KIND, int L, int C, bool KSMEM, bool TRAJ, bool NOISE, bool UNITS>
-static void launch_tick(const TickArgs& a, int grid, int block, size_t smem, cudaStream_t st) {
-  launch_dependent(tick_kernel<KIND, L, C, KSMEM, TRAJ, false, NOISE, UNITS>, grid, block, smem, st,
-                   a);
+static void launch_tick(const TickArgs& a, int grid, int block, size_t smem, cudaStream_t st,
+                        bool early) {
+  launch_early(early, tick_kernel<KIND, L, C, KSMEM, TRAJ, false, NOISE, UNITS>, grid, block, smem,
+               st, a);
 }
 
 template <int KIND, int L, int C, bool KSMEM, bool TRAJ, bool NOISE>
