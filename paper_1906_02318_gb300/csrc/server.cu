@@ -93,7 +93,9 @@ __device__ __forceinline__ void fold_take(const SessionTick& st, unsigned long l
   sc->done = 0u;
 }
 
-template <int KIND, int L, int C, bool KSMEM>
+// UNITS: the blocks take sorted units (one lane); an instance of its own, since small
+// batches paid 2 us for the code beside theirs.
+template <int KIND, int L, int C, bool KSMEM, bool UNITS>
 __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_constant__ ServeArgs sa) {
   using B = BasisTraits<KIND>;
   constexpr int N = B::N, NX = B::NX, NU = B::NU;
@@ -111,8 +113,8 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
   // staging anything, so that a small batch holds few SMs and batches in flight at the
   // same time share the device
   ServeHeader* hdr = sa.table;
-  const int total = hdr->total, unit = hdr->unit, n_req = hdr->n_requests;
-  if ((long long)blockIdx.x * (unit ? 1 : blockDim.x >> 5) >= (long long)total) return;
+  const int total = hdr->total, n_req = hdr->n_requests;
+  if ((long long)blockIdx.x * (UNITS ? 1 : blockDim.x >> 5) >= (long long)total) return;
 
   if constexpr (PK) {
     const uint4* src = reinterpret_cast<const uint4*>(sa.Kp);
@@ -168,16 +170,16 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
     if constexpr (ANG >= 0) sincosf(xs[ANG], &sn, &cs);
     cur = req;
   };
-  if (unit == 0) {
+  if constexpr (!UNITS) {
     const int wpb = blockDim.x >> 5;
     for (int gwt = blockIdx.x * wpb + warp; gwt < total; gwt += gridDim.x * wpb) {
-      const int r = range_of(gwt), req = ent[r].range_entry;
+      const int req = range_of(gwt);  // tiles come in the order of the requests
       const SessionTick& st = ent[req];
       load_state(st, req);
       unsigned long long best = ~0ull;
       unsigned int n_safe = 0, n_exec = 0;
-      run_tile<KIND, L, C, KSMEM, false, false, true, false>(
-          st, dyn_of(st), sa.safety, gwt - ent[r].range_begin, st.n_slots, xs, uh, sn, cs, kr, sK4,
+      run_tile<KIND, L, C, KSMEM, false, false, true, (L > 1)>(
+          st, dyn_of(st), sa.safety, gwt - st.range_begin, st.n_slots, xs, uh, sn, cs, kr, sK4,
           tv, &s_x[L > 1 ? warp : 0][0][0][0], best, n_safe, n_exec);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
@@ -189,9 +191,8 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
       if (lane == 0) fold_take<NU>(st, best, ((unsigned long long)n_safe << 40) + n_exec, uh);
       __syncwarp();
     }
-    return;
-  }
-  if constexpr (L == 1) {
+  } else {
+    const int unit = hdr->unit;
     char* buf = reinterpret_cast<char*>(s_dyn + KWORDS) +
                 (B::TRACK && sa.safety.has_track ? sa.safety.track.blob_bytes : 0);
     __shared__ int s_unit, s_tile;
@@ -247,21 +248,28 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
 struct ServeKernel {
   const void* fn = nullptr;
   void (*launch)(const ServeArgs&, int, int, size_t, cudaStream_t) = nullptr;
+  // the same shape over sorted units (one lane)
+  const void* fn_units = nullptr;
+  void (*launch_units)(const ServeArgs&, int, int, size_t, cudaStream_t) = nullptr;
   size_t k_smem = 0;
   int per_warp = 32;
   int lanes = 1, cands = 1;
 };
 
-template <int KIND, int L, int C, bool KSMEM>
+template <int KIND, int L, int C, bool KSMEM, bool UNITS>
 static void launch_serve(const ServeArgs& a, int grid, int block, size_t smem, cudaStream_t st) {
-  serve_kernel<KIND, L, C, KSMEM><<<grid, block, smem, st>>>(a);
+  serve_kernel<KIND, L, C, KSMEM, UNITS><<<grid, block, smem, st>>>(a);
 }
 
 template <int KIND, int L, int C, bool KSMEM>
 static ServeKernel make_serve() {
   ServeKernel k;
-  k.fn = reinterpret_cast<const void*>(&serve_kernel<KIND, L, C, KSMEM>);
-  k.launch = &launch_serve<KIND, L, C, KSMEM>;
+  k.fn = reinterpret_cast<const void*>(&serve_kernel<KIND, L, C, KSMEM, false>);
+  k.launch = &launch_serve<KIND, L, C, KSMEM, false>;
+  if constexpr (L == 1) {
+    k.fn_units = reinterpret_cast<const void*>(&serve_kernel<KIND, L, C, KSMEM, true>);
+    k.launch_units = &launch_serve<KIND, L, C, KSMEM, true>;
+  }
   k.k_smem = (size_t)ksmem_words<KIND, L, KSMEM, true>() * 16;
   k.per_warp = 32 / L * C;
   k.lanes = L;
@@ -287,22 +295,43 @@ static std::vector<ServeKernel> serve_shapes(int kind) {
   return {};
 }
 
-// The shape an untuned server takes for batches of at least kLargeBatch slots per SM: two
-// race cars per thread, so that a word of K from shared memory, which bounds the one-lane
-// step, serves two predictions, in blocks of 256.  Race cars, N and H as in plan_batch,
-// submit to collect, one candidate per thread against two: 12 sessions (fewer slots than
-// that) 460 against 425 us alone but 513 against 564 with balance bots beside them, 16
-// sessions 604 against 529, 24 698 against 616, 60 1853 against 1575.  The balance bot
-// keeps K in registers and gains nothing.
-constexpr int kLargeBatch = 1200;
-static ServeKernel large_serve(int kind) {
-  return kind == kCar ? make_serve<kCar, 1, 2, true>() : ServeKernel{};
+// The shapes an untuned server takes instead of the initial one, and which of them
+// (-1: the initial one) a batch of that many slots takes.
+//
+// Large batches: two race cars per thread, so that a word of K from shared memory, which
+// bounds the one-lane step, serves two predictions, in blocks of 256.  Race cars, N and
+// H as in plan_batch, submit to collect, one candidate per thread against two: 12
+// sessions (fewer than 1,200 slots per SM) 460 against 425 us alone but 513 against 564
+// with balance bots beside them, 16 sessions 604 against 529, 24 698 against 616, 60
+// 1853 against 1575.
+//
+// Small race-car batches: several lanes per candidate, as a single tick of that size
+// takes, since one lane's step takes 1.7 us however few there are: one session, H = 60,
+// N = 1000 103 -> 65 us and N = 3000 103 -> 69 with eight lanes, N = 6000 102 -> 78 and N =
+// 18000 135 -> 99 with two.  Two lanes gain again from 256 to 512 slots per SM (277 -> 206,
+// 281 -> 229), but not between (131 -> 136, 176 -> 160, 181 -> 188) nor past it (271 ->
+// 290).  The balance bot gains from neither (four lanes, N = 1000: 46 -> 48).
+struct ServeAlt {
+  ServeKernel kern;
+  int block;
+};
+static std::vector<ServeAlt> serve_alts(int kind) {
+  if (kind == kCar)
+    return {{make_serve<kCar, 8, 1, false>(), 128},
+            {make_serve<kCar, 2, 1, true>(), 128},
+            {make_serve<kCar, 1, 2, true>(), 256}};
+  return {};
+}
+static int pick_alt(int kind, long long slots, int sms) {
+  if (kind != kCar) return -1;
+  if (slots < 32LL * sms) return 0;
+  if (slots < 128LL * sms || (slots >= 256LL * sms && slots < 512LL * sms)) return 1;
+  return slots >= 1200LL * sms ? 2 : -1;
 }
 
-// Dynamic shared memory of a shape: K, the track grid, and a sorted unit.
+// Dynamic shared memory of a shape: K and the track grid (a sorted unit on top).
 static size_t serve_smem(const ServeKernel& k, const DevSafety& safety) {
-  return k.k_smem + (safety.has_track ? (size_t)safety.track.blob_bytes : 0) +
-         (k.lanes == 1 ? unit_bytes(kServeUnit) : 0);
+  return k.k_smem + (safety.has_track ? (size_t)safety.track.blob_bytes : 0);
 }
 
 static ServeKernel pick_serve(int kind) {
@@ -317,12 +346,13 @@ constexpr int kServeBuffers = 5;                      // batch buffers
 constexpr int kServeMaxInFlight = kServeBuffers - 1;  // one is always free for staging
 
 namespace mpmi {
-// A launch shape of the server with its captured graphs, one per batch buffer.
+// A launch shape of the server with its captured graphs, one per batch buffer, over
+// tiles [0] and over sorted units [1] (one-lane shapes).
 struct ServeShape {
   ServeKernel kern;
-  int grid = 0, block = 128;
-  size_t smem = 0;
-  cudaGraphExec_t graph[kServeBuffers] = {};
+  int block = 128;
+  int grid[2] = {};
+  cudaGraphExec_t graph[2][kServeBuffers] = {};
 };
 }  // namespace mpmi
 
@@ -353,7 +383,7 @@ struct mpmi_server {
   int max_in_flight = kServeMaxInFlight;
   size_t table_bytes = 0;
   mpmi::ServeShape shape;  // the initial or tuned one
-  mpmi::ServeShape large;  // untuned servers: for large batches (no kernel: none)
+  std::vector<mpmi::ServeShape> alts;  // untuned servers: serve_alts, by the batch's size
   uint64_t per_session_bytes = 0, bytes = 0;
 };
 
@@ -368,7 +398,7 @@ static int sfail(cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return sfail(e_, what); \
   } while (0)
 
-static int build_graph(mpmi_server* s, ServeShape& shape, int b) {
+static int build_graph(mpmi_server* s, ServeShape& shape, int units, int b) {
   ServeArgs a;
   memset(&a, 0, sizeof(a));
   a.K = s->model->K32_dev;
@@ -376,16 +406,19 @@ static int build_graph(mpmi_server* s, ServeShape& shape, int b) {
   a.Kp = s->model->K32_dev + 2 * (size_t)s->model->n * s->model->n;
   a.safety = s->model->dev_safety;
   a.table = s->table_dev[b];
+  const size_t smem =
+      serve_smem(shape.kern, s->model->dev_safety) + (units ? unit_bytes(kServeUnit) : 0);
   cudaGraph_t g = nullptr;
   SRV_CUDA(cudaStreamBeginCapture(s->capture, cudaStreamCaptureModeThreadLocal), "begin capture");
   cudaMemcpyAsync(s->table_dev[b], s->table_host[b], s->table_bytes, cudaMemcpyHostToDevice,
                   s->capture);
-  shape.kern.launch(a, shape.grid, shape.block, shape.smem, s->capture);
+  (units ? shape.kern.launch_units : shape.kern.launch)(a, shape.grid[units], shape.block, smem,
+                                                        s->capture);
   cudaMemcpyAsync(s->res_host[b], s->res_dev[b], sizeof(mpmi_result) * s->max_sessions,
                   cudaMemcpyDeviceToHost, s->capture);
   cudaError_t e = cudaStreamEndCapture(s->capture, &g);
   if (e != cudaSuccess) return sfail(e, "end capture");
-  e = cudaGraphInstantiate(&shape.graph[b], g, 0);
+  e = cudaGraphInstantiate(&shape.graph[units][b], g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) return sfail(e, "graph instantiate");
   return MPMI_OK;
@@ -399,28 +432,30 @@ static int build_graph(mpmi_server* s, ServeShape& shape, int b) {
 // way).  Mixed sizes and horizons (N log-uniform in 1k..64k, H in 20..100), untuned
 // servers, one candidate per thread, submit to collect: 24 race cars 850 -> 702 us, 60
 // 2320 -> 1860; 24 balance bots 210 -> 168, 60 455 -> 336; both servers together, 48
-// sessions 1077 -> 806 (713 with large_serve's shape).  One to six units per block measured the same within 2 % from two on.
+// sessions 1077 -> 806 (713 with two race cars per thread).  One to six units per block
+// measured the same within 2 % from two on.
 // Returns the shape to launch.
 static const ServeShape& plan_batch(const mpmi_server* s, ServeHeader* hdr) {
   SessionTick* ent = reinterpret_cast<SessionTick*>(hdr + 1);
   const int n = hdr->n_requests;
   long long slots = 0;
   for (int i = 0; i < n; ++i) slots += ent[i].n_slots;
-  const ServeShape& shape =
-      s->large.kern.fn != nullptr && slots >= (long long)kLargeBatch * s->ctx->sm_count ? s->large
-                                                                                       : s->shape;
+  const int alt = pick_alt(s->model->kind, slots, s->ctx->sm_count);
+  const bool other = alt >= 0 && alt < (int)s->alts.size() && s->alts[alt].kern.fn != nullptr;
+  const ServeShape& shape = other ? s->alts[alt] : s->shape;
   const ServeKernel& k = shape.kern;
   std::vector<int> by(n);
   for (int i = 0; i < n; ++i) by[i] = i;
-  const long long warps = (long long)shape.grid * (shape.block / 32);
+  const int grid = shape.grid[1];  // 0: no sorted units
+  const long long warps = (long long)grid * (shape.block / 32);
   const int min_tiles = s->model->kind == kCar ? 2 : 4;  // per warp
   hdr->unit = 0;
-  if (k.lanes == 1 && slots >= min_tiles * warps * k.per_warp) {
+  if (grid > 0 && slots >= min_tiles * warps * k.per_warp) {
     std::stable_sort(by.begin(), by.end(),
                      [&](int a, int b) { return ent[a].horizon > ent[b].horizon; });
     // a multiple of one tile per warp of a block, about three units per block
     const int step = k.per_warp * (shape.block / 32);
-    const long long want = slots / (3LL * shape.grid);
+    const long long want = slots / (3LL * grid);
     hdr->unit = (int)std::min<long long>(kServeUnit / step,
                                          std::max<long long>(1, (want + step / 2) / step)) * step;
   }
@@ -445,15 +480,16 @@ static int n_flying(const mpmi_server* s) {
 }
 
 static void drop_graphs(ServeShape& shape) {
-  for (cudaGraphExec_t& g : shape.graph) {
-    if (g) cudaGraphExecDestroy(g);
-    g = nullptr;
-  }
+  for (auto& graphs : shape.graph)
+    for (cudaGraphExec_t& g : graphs) {
+      if (g) cudaGraphExecDestroy(g);
+      g = nullptr;
+    }
 }
 
 static void server_release_device(mpmi_server* s) {
   drop_graphs(s->shape);
-  drop_graphs(s->large);
+  for (ServeShape& z : s->alts) drop_graphs(z);
   for (int b = 0; b < kServeBuffers; ++b) {
     for (cudaEvent_t e : {s->start[b], s->done[b], s->after[b]})
       if (e) cudaEventDestroy(e);
@@ -472,26 +508,28 @@ static void server_release_device(mpmi_server* s) {
 // the shape cannot be resident (the record keeps what it had).
 static int server_set_shape(mpmi_server* s, ServeShape& shape, const ServeKernel& k, int block) {
   const size_t smem = serve_smem(k, s->model->dev_safety);
-  if (smem > 0 &&
-      cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return fail(MPMI_E_UNSUPPORTED, "server: shape cannot take its shared memory");
+  int nb[2] = {};
+  for (int units = 0; units < (k.fn_units ? 2 : 1); ++units) {
+    const void* fn = units ? k.fn_units : k.fn;
+    const size_t bytes = smem + (units ? unit_bytes(kServeUnit) : 0);
+    if ((bytes > 0 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)bytes) != cudaSuccess) ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb[units], fn, block, bytes) !=
+            cudaSuccess) {
+      cudaGetLastError();
+      nb[units] = 0;
+    }
   }
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn, block, smem) != cudaSuccess ||
-      nb < 1) {
-    cudaGetLastError();
-    return fail(MPMI_E_UNSUPPORTED, "server: shape cannot be resident");
-  }
+  if (nb[0] < 1) return fail(MPMI_E_UNSUPPORTED, "server: shape cannot be resident");
   drop_graphs(shape);
   shape.kern = k;
   shape.block = block;
-  shape.smem = smem;
-  shape.grid = nb * s->ctx->sm_count;
-  for (int b = 0; b < kServeBuffers; ++b) {
-    const int rc = build_graph(s, shape, b);
-    if (rc != MPMI_OK) return rc;
+  for (int units = 0; units < 2; ++units) {
+    shape.grid[units] = nb[units] * s->ctx->sm_count;
+    for (int b = 0; b < kServeBuffers && shape.grid[units] > 0; ++b) {
+      const int rc = build_graph(s, shape, units, b);
+      if (rc != MPMI_OK) return rc;
+    }
   }
   return MPMI_OK;
 }
@@ -555,12 +593,11 @@ int mpmi_server_create(mpmi_ctx* ctx, const mpmi_model* model, int32_t max_sessi
     cudaMemset(s->table_dev[b], 0, s->table_bytes);
   }
   int rc = server_set_shape(s, s->shape, kern, 128);
-  if (rc == MPMI_OK && large_serve(model->kind).fn != nullptr) {
-    rc = server_set_shape(s, s->large, large_serve(model->kind), 256);
-    if (rc == MPMI_E_UNSUPPORTED) {  // every batch takes the initial shape
-      s->large = ServeShape{};
-      rc = MPMI_OK;
-    }
+  for (const ServeAlt& alt : serve_alts(model->kind)) {
+    if (rc != MPMI_OK) break;
+    s->alts.emplace_back();
+    rc = server_set_shape(s, s->alts.back(), alt.kern, alt.block);
+    if (rc == MPMI_E_UNSUPPORTED) rc = MPMI_OK;  // such batches take the initial shape
   }
   if (rc != MPMI_OK) {
     server_release_device(s);
@@ -700,7 +737,8 @@ int mpmi_server_launch(mpmi_server* s, void* stream, int32_t* n_launched) {
   SRV_CUDA(cudaEventRecord(s->after[b], st), "server event");
   SRV_CUDA(cudaStreamWaitEvent(s->bstream[b], s->after[b], 0), "server stream wait");
   SRV_CUDA(cudaEventRecord(s->start[b], s->bstream[b]), "server event");
-  SRV_CUDA(cudaGraphLaunch(shape.graph[b], s->bstream[b]), "server graph launch");
+  SRV_CUDA(cudaGraphLaunch(shape.graph[s->table_host[b]->unit ? 1 : 0][b], s->bstream[b]),
+           "server graph launch");
   SRV_CUDA(cudaEventRecord(s->done[b], s->bstream[b]), "server event");
   if (n_launched) *n_launched = n;
   s->flying[b] = true;
@@ -818,8 +856,8 @@ int mpmi_server_tune(mpmi_server* s, int32_t n, const mpmi_session_config* cfgs,
   std::vector<float> t(reps);
   const ServeKernel initial = s->shape.kern;
   const int initial_block = s->shape.block;
-  const ServeShape large = s->large;  // every batch takes the shape being timed
-  s->large = ServeShape{};
+  std::vector<ServeShape> alts;  // every batch takes the shape being timed
+  alts.swap(s->alts);
   ServeKernel best_k = initial;
   int best_block = initial_block;
   mpmi_tune_result best;
@@ -872,10 +910,10 @@ int mpmi_server_tune(mpmi_server* s, int32_t n, const mpmi_session_config* cfgs,
   // keep the winner (or go back to the initial shape after a failure)
   const int rc2 = server_set_shape(s, s->shape, rc == MPMI_OK ? best_k : initial,
                                    rc == MPMI_OK ? best_block : initial_block);
-  s->large = large;
   if (rc == MPMI_OK) {  // a tuned server keeps to its winner
-    drop_graphs(s->large);
-    s->large = ServeShape{};
+    for (ServeShape& z : alts) drop_graphs(z);
+  } else {
+    s->alts.swap(alts);
   }
   release_all();
   if (rc != MPMI_OK) return rc;

@@ -141,3 +141,11 @@ def test_samples_in_order(setup, which, N):
     _same(*out)
     assert np.mean(f["ttv"] != out[0]["ttv"]) < 1e-3
     assert np.array_equal(f["cost"], out[0]["cost"])
+
+
+@pytest.mark.parametrize("which,sizes", [
+    ("car", [(3001, 30), (0, 60), (33, 25)]), ("car", [(9001, 60), (4096, 25), (257, 100)]),
+    ("car", [(40001, 30), (9999, 60), (1, 20)]), ("bot", [(2001, 50), (0, 20), (77, 100)])])
+def test_served_small_batches_equal_the_tick_alone(setup, which, sizes):
+    """Batches of the sizes at which an untuned server takes several lanes per candidate."""
+    test_served_units_equal_the_tick_alone(setup, which, sizes)
