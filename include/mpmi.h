@@ -161,7 +161,8 @@ uint64_t mpmi_memory_in_use(const mpmi_ctx* ctx);
  *   K = argmin sum_m || Psi(x_next[m], u[m]) - K Psi(x[m], u[m]) ||^2
  * x, x_next: m x nx row-major; u: m x nu row-major (the input is held over the
  * step, so the target lifts x_next with the same u).  Solved by Householder QR
- * in float64 on the host (an offline step, Sec. IV-A "learned offline").
+ * in float64 on the host, row blocks on several threads (an offline step, Sec. IV-A
+ * "learned offline"); the result does not depend on the number of threads.
  * *residual_out (may be NULL) = ||X K^T - Y||_F / ||Y||_F.  The model's device
  * copy of K is float32 (round to nearest).  Fails with INVALID_ARG when m < n,
  * NONFINITE on NaN/Inf input, and INVALID_ARG if the lifted data is rank
@@ -420,7 +421,8 @@ int mpmi_debug_trajectories(mpmi_session* s, const double* x_t_dev,
 /* Serves many control sessions of one model together: each admitted session has
  * its own N, H, input box, sampler seed/stream and tick counter; the requests
  * staged for a batch run in one launch (replayed from a CUDA graph) whose warps
- * stride over all requests' candidates, and every request's result is
+ * take tiles of all requests' candidates (the launch shape and, in large batches,
+ * the candidates' order depend on the batch), and every request's result is
  * bit-identical to the same tick evaluated alone (same per-candidate arithmetic,
  * exact min-reduction).  Up to four batches of the server run at once, each on a
  * stream of the server's own, while the requests of the next one are staged on

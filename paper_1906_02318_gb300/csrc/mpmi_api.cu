@@ -321,8 +321,8 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
   if (small) small_shape(s->model->kind, list_lanes, &lanes, &cands, &block);
   const bool noise = a.n_noise > 0;
   // noisy balance-bot ticks: four lanes draw four steps' noise at once, which pays up to
-  // 2.5 four-lane warps per SM sub-partition (N = 10000 20.9 us against 23.0 with one
-  // lane, N = 16384 27.0 against 22.9)
+  // 2.5 four-lane warps per SM sub-partition (N = 10000 18.5 us against 19.7 with one
+  // lane, N = 12000 18.7 against 22.1, N = 16384 23.9 against 23.7)
   if (noise && !small && s->auto_lanes && lanes == 1 && s->model->kind == kBot &&
       s->n_slots <= 80 * s->ctx->sm_count)
     lanes = 4;

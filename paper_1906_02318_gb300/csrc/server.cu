@@ -11,8 +11,8 @@
 // served alone or in a mix.
 //
 // Host side: admission (a free session slot and room in the context's memory
-// budget), kBuffers batch buffers, each with one captured graph (table upload,
-// kernel, result download) and a stream of its own, so a batch costs one graph
+// budget), kServeBuffers batch buffers, each with a captured graph per launch shape
+// (table upload, kernel, result download) and a stream of its own, so a batch costs one graph
 // launch and up to max_in_flight batches of the model run at once while the
 // requests for the next one are staged.  A session has at most one request
 // staged or on the GPU, so batches in flight touch disjoint reduction records;

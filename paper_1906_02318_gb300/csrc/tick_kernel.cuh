@@ -883,8 +883,9 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
   // every step's before), and one lane with K in registers draws four, their chains
   // side by side (the race car's one-lane shapes have no registers left for that).
   // Normals past the horizon are drawn and not used.  GB300: balance bot H = 50,
-  // N = 1000 (4 lanes) 27.3 -> 15 us, N = 16384 (1 lane) 27.1 -> 22.9; race car H = 60,
-  // N = 1024 (16 lanes) 60 -> 30 us, N = 4096 (8) 76 -> 44, N = 16384 (2) 97 -> 80.
+  // N = 1000 (4 lanes) 27.3 -> 12 us, N = 16384 (1 lane) 27.1 -> 23.7; race car H = 60,
+  // N = 1024 (16 lanes) 60 -> 24 us, N = 4096 (8) 76 -> 36, N = 16384 (2) 97 -> 72 (the
+  // launches' early start is 2 to 3 us of each).
   constexpr int AHEAD = !NOISE ? 1 : (L > 1 ? L : (KIND != kCar && C == 1 ? 4 : 1));
   float ahead[AHEAD >= L ? AHEAD / L : 1][NX];
   // z <- K z, then the step's noise
