@@ -149,3 +149,24 @@ def test_samples_in_order(setup, which, N):
 def test_served_small_batches_equal_the_tick_alone(setup, which, sizes):
     """Batches of the sizes at which an untuned server takes several lanes per candidate."""
     test_served_units_equal_the_tick_alone(setup, which, sizes)
+
+
+def test_tensor_rollout_one_or_several_tiles_per_cta(setup):
+    """Either side of the size at which the tensor-core rollout's CTAs take more than one
+    tile (another kernel instance): the candidates both ticks share agree bit for bit."""
+    import torch
+    lib, ctx, envs = setup
+    env, model = envs["car"]
+    tiles = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    x_t = data.car_start_state(env.track, vx=14.0) + np.array([0.5, -0.5, 0.1, 0, 0, 0])
+    u_h = data.to_f32_exact(data.user_input_once(9, env.lo, env.hi))
+    out = []
+    for n_slots in (128 * tiles, 128 * tiles + 1):
+        s = lib.Session(ctx, model, n_slots - 1, 60, env.lo, env.hi, seed=11)
+        s.set_rollout("tensor")
+        out.append(run_gpu(lib, s, x_t, u_h, tick=3))
+        s.close()
+    n = 128 * tiles
+    assert np.array_equal(out[0]["ttv"], out[1]["ttv"][:n])
+    assert np.array_equal(out[0]["cost"], out[1]["cost"][:n])
+    assert 0 < out[0]["result"]["n_safe"] < n
