@@ -98,11 +98,14 @@ struct TrainSmem {
   static constexpr int BYTES = FLOATS * 4;
 };
 
+// Launched early, so the kernels that write P (the Adam update of the step before), feats
+// and target may still run when it starts: plain loads behind the wait, never the
+// read-only path (__ldg, const __restrict__), which holds only for data that nothing
+// writes while the kernel is resident.  The same goes for part in reduce_grad.
 template <int SPT>
-__global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(const float* __restrict__ P,
-                                                                const float* __restrict__ feats,
-                                                                const float* __restrict__ target,
-                                                                int B, float* __restrict__ part) {
+__global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(const float* P, const float* feats,
+                                                                const float* target, int B,
+                                                                float* part) {
   using S = TrainSmem<SPT>;
   constexpr int T = S::T;
   extern __shared__ __align__(16) float sm[];
@@ -120,13 +123,13 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(const float* __r
   if (tid == 0) bar_expect(&s_bar, kH * kH * 4);
   __syncthreads();
   if (tid < kH) bulk_g2s(sW2 + tid * kRow, P + oW2 + tid * kH, kH * 4, &s_bar);
-  for (int i = tid; i < kH * kIn; i += kTrainThreads) sW1[i] = __ldg(P + oW1 + i);
+  for (int i = tid; i < kH * kIn; i += kTrainThreads) sW1[i] = P[oW1 + i];
   if (tid < kH) {
-    sb1[tid] = __ldg(P + ob1 + tid);
-    sb2[tid] = __ldg(P + ob2 + tid);
-    sw3[tid] = __ldg(P + ow3 + tid);
+    sb1[tid] = P[ob1 + tid];
+    sb2[tid] = P[ob2 + tid];
+    sw3[tid] = P[ow3 + tid];
   }
-  float b3 = __ldg(P + ob3);
+  float b3 = P[ob3];
   const float scale = 2.f / (float)B;
 
   float gW2[8][8];  // rows 4 sg + a, 64 + 4 sg + a; columns 4 jg + c, 64 + 4 jg + c
@@ -147,7 +150,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(const float* __r
 #pragma unroll
     for (int i = 0; i < SPT; ++i) {
       const int s = sg * SPT + i;
-      tv[i] = s < live ? __ldg(target + s0 + s) : 0.f;
+      tv[i] = s < live ? target[s0 + s] : 0.f;
     }
     __syncthreads();
     // layer 1, units jg + 16 e of samples sg SPT + i
@@ -339,14 +342,13 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(const float* __r
 }
 
 // Adds the blocks' records: eight threads per parameter take every eighth record, in
-// order, all of a thread's loads in flight.  With lr > 0 the sum feeds Adam (params, m, v updated in place), else it is
-// stored in grad.  The value after the parameters is the loss.
+// order, all of a thread's loads in flight.  With lr > 0 the sum feeds Adam (params, m, v
+// updated in place), else it is stored in grad.  The value after the parameters is the
+// loss.
 constexpr int kRedParams = 64, kRedSlices = 8;
-__global__ void __launch_bounds__(kRedSlices * kRedParams) reduce_grad(const float* __restrict__ part,
-                                                             int n_part, int B, float* grad,
-                                                             float* loss, float* P, float* m,
-                                                             float* v, float lr, float c1,
-                                                             float c2) {
+__global__ void __launch_bounds__(kRedSlices * kRedParams)
+    reduce_grad(const float* part, int n_part, int B, float* grad, float* loss, float* P, float* m,
+                float* v, float lr, float c1, float c2) {
   __shared__ float s[kRedSlices][kRedParams];
   const int x = threadIdx.x % kRedParams, y = threadIdx.x / kRedParams;
   const int i = blockIdx.x * kRedParams + x;

@@ -110,3 +110,40 @@ def test_host_ticks_alternate_streams(setup):
         s.close()
         out.append(got)
     assert out[0] == out[1] == out[2]
+
+
+def test_training_steps_back_to_back(setup):
+    """Training steps with nothing between them but the kernel that gathers the next
+    minibatch: the losses and weights of the same steps with a wait after each."""
+    import torch
+    lib, ctx, envs = setup
+    model = envs["car"][1]
+    rng = np.random.default_rng(12)
+    bank = torch.tensor(rng.uniform(-1, 1, (20000, 12)), dtype=torch.float32, device="cuda")
+    target = torch.tensor(rng.uniform(0, 1, 20000), dtype=torch.float32, device="cuda")
+    sizes = [256, 17, 4096, 8192, 2500] * 10
+    pick = [torch.tensor(rng.integers(0, 20000, b), device="cuda") for b in sizes]
+    out = []
+    for wait in (True, False):
+        scr = lib.Screener(ctx, model, data.screener_init(7), max_batch=8192, max_slots=64)
+        loss = torch.zeros(len(sizes), device="cuda")
+        grad = torch.zeros((len(sizes), lib.SCREENER_PARAMS), device="cuda")
+        f, y = torch.empty((8192, 12), device="cuda"), torch.empty(8192, device="cuda")
+        scr.train_step(bank[:64], target[:64], loss[:1])  # all buffers and code are in place
+        torch.cuda.synchronize()
+        for t, i in enumerate(pick):
+            torch.index_select(bank, 0, i, out=f[:len(i)])
+            torch.index_select(target, 0, i, out=y[:len(i)])
+            if t % 3 == 2:
+                scr.gradients(f[:len(i)], y[:len(i)], grad[t], loss[t:t + 1])
+            scr.train_step(f[:len(i)], y[:len(i)], loss[t:t + 1], lr=1e-2)
+            scr.train_step(f[:len(i)], y[:len(i)], loss[t:t + 1], lr=1e-2)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        w = lib.pack_weights(scr.get_weights())
+        out.append((loss.cpu().numpy(), grad.cpu().numpy(), w))
+        scr.free()
+    assert np.all(np.isfinite(out[0][0])) and len(set(out[0][0])) > 40
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
