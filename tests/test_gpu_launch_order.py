@@ -147,3 +147,54 @@ def test_training_steps_back_to_back(setup):
     assert np.all(np.isfinite(out[0][0])) and len(set(out[0][0])) > 40
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("rollout", ["full", "tensor", "factored"])
+def test_screened_ticks_back_to_back(setup, rollout):
+    """Screened ticks in cost order and with the network, some falling back to the full
+    evaluation, between training steps (the network's weights change under way) and on
+    states that a kernel on the stream writes: the same ticks with a wait after each."""
+    import torch
+    lib, ctx, envs = setup
+    env, model = envs["car"]
+    N, T = 3000, 36
+    rng = np.random.default_rng(21)
+    x0 = data.car_start_state(env.track, vx=12.0)
+    bank = x0 + rng.uniform(-1, 1, (T, 6)) * [1.5, 1.5, 0.2, 4, 0.3, 0.3]
+    bank[::5, :2] += 40.0  # off the road: every kept slot is unsafe
+    bank = torch.tensor(bank, device="cuda")
+    u = torch.tensor(data.to_f32_exact(data.user_input_once(2, env.lo, env.hi)), device="cuda")
+    f = torch.tensor(rng.uniform(-1, 1, (512, 12)), dtype=torch.float32, device="cuda")
+    y = torch.tensor(rng.uniform(0, 1, 512), dtype=torch.float32, device="cuda")
+    idx = [torch.tensor([t], device="cuda") for t in range(T)]
+    w = {k: np.asarray(v).copy() for k, v in data.screener_init(7).items()}
+    w["w3"] = (4.0 * w["w3"]).astype(np.float32)  # spread the scores
+    out = []
+    for wait in (True, False):
+        scr = lib.Screener(ctx, model, w, max_batch=512, max_slots=N + 1)
+        s = lib.Session(ctx, model, N, 40, env.lo, env.hi, seed=3)
+        s.set_rollout(rollout)
+        x = torch.zeros((1, 6), dtype=torch.float64, device="cuda")
+        loss = torch.zeros(T, device="cuda")
+        res = torch.zeros((T, lib.RESULT_BYTES), dtype=torch.uint8, device="cuda")
+        lst = torch.full((T, N + 1), -1, dtype=torch.int32, device="cuda")
+        cnt = torch.zeros((T, 1), dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        for t in range(T):
+            torch.index_select(bank, 0, idx[t], out=x)
+            tau, k = [(0.0, 150), (0.5, 1), (0.9, 1)][t % 3]
+            lists = dict(list_dev=lst[t], n_list_dev=cnt[t]) if t % 4 == 3 else {}
+            lib.evaluate_screened(s, scr, x[0], u, res[t], k=k, tau=tau, m=16, tick=t, **lists)
+            if t % 6 == 5:
+                scr.train_step(f, y, loss[t:t + 1], lr=1e-2)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        kept = [sorted(row[:n].tolist()) for row, n in zip(lst.cpu().numpy(), cnt.cpu().numpy()[:, 0])]
+        out.append((res.cpu().numpy(), loss.cpu().numpy(), kept))
+        s.close()
+        scr.free()
+    flags = [lib.result_from_bytes(torch.from_numpy(r), 2)["flags"] for r in out[0][0]]
+    assert any(g & 2 for g in flags) and any(not g & 2 for g in flags)
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+    assert out[0][2] == out[1][2] and any(out[0][2])
