@@ -1,0 +1,67 @@
+// Rules on sizes that the tick launches follow, with the measurements behind them (GB300,
+// 152 SMs, ticks back to back, eight states of a closed loop).  Plain host code, so that
+// the lines can be checked without a GPU.
+#pragma once
+
+#include "basis.h"
+
+namespace mpmi {
+
+// Horizon from which a tick of S/2 < blocks <= S keeps the stream's order instead of
+// starting early (S: SMs).  While the blocks of the tick before hold their SMs, an early
+// grid doubles up on the idle ones; an early start gives about 2 us whatever the horizon,
+// and two blocks on an SM slow each other down in every step.  How many pair up settles
+// differently from run to run (both modes given where they were seen), so the lines lie
+// where the slower one no longer loses much.  In order / early, us:
+//   race car, K in shared memory (two lanes), 110 blocks: H = 20 16.6 / 14.3, 30 20.7 /
+//     19.5 (79 blocks 18.6 or 24.7), 40 26.2 / 28.3, 60 36.5 / 41.5, 100 53.5 / 64.8;
+//     noisy, 79 to 110 blocks, H = 20 22.7 / 20.5 or 25.0, 30 30.7 / 32.0, 60 53.6 / 60.9
+//   eight lanes, 96 blocks: H = 60 20.6 / 18.1, 70 22.7 / 23.0, 100 28.5 / 32.1; noisy, H
+//     = 40 20.6 / 19.3, 60 26.8 / 25.0, 70 30.0 / 32.7; 126 blocks: H = 40 16.6 / 14.3, 60
+//     20.6 / 18.2 or 22.4, 70 22.7 / 23.5; noisy, H = 30 18.6 / 16.2, 40 22.1 / 22.7, 100
+//     39.1 / 44.9
+//   sixteen lanes, 96 blocks: H = 60 18.4 / 17.4, 80 20.7 / 21.7, 100 24.7 / 25.9; noisy,
+//     H = 50 18.6 / 18.1, 60 20.7 / 21.3, 100 30.7 / 32.5
+//   balance bot, one lane, 84 to 140 blocks: H = 60 10.5 / 8.5 to 10.8, 80 12.4 / 10.1 or
+//     13.6, 90 12.5 / 13.7, 100 14.4 / 14.9; noisy, H = 30 16.3 / 15.9, 40 18.6 / 19.4, 100
+//     37.0 / 40.9; noisy, four lanes, 124 blocks: H = 70 18.1 / 17.7, 80 18.6 / 19.7, 100
+//     22.7 / 24.3
+// On every SM but a few (152 blocks) the balance bot loses earlier: one lane, H = 50 10.3
+// / 10.4, 60 10.4 / 12.1, 100 14.4 / 17.6.  Its four lanes without noise never do.
+inline int order_horizon(int kind, int lanes, bool k_shared, bool noise, long long grid, int sms) {
+  constexpr int kNever = 1 << 30;
+  if (kind == kCar) {
+    if (k_shared) return noise ? 0 : 25;
+    if (lanes == 16) return noise ? 55 : 75;
+    return 4 * grid > 3LL * sms ? (noise ? 35 : 45) : (noise ? 50 : 65);
+  }
+  if (kind != kBot || (lanes > 1 && !noise)) return kNever;
+  const int h = lanes > 1 ? 78 : (noise ? 35 : 75);
+  return 100 * grid > 97LL * sms ? h * 2 / 3 : h;
+}
+
+// Whether a launch keeps the stream's order: `grid` of at most `resident` blocks with
+// `warps_per_block` warps each over `tiles` warp-tiles, taken in strides (not sorted units).
+//
+// With more tiles than resident warps the first blocks take a tile more.  In order they
+// spread over the SMs; early they start two to an SM as it falls free, and where the last
+// round holds between a fifth and 3/8 of a round, those pairs take as long as a full
+// round.  Race car, two candidates per thread, in order / early, us: N = 98558 (27 % of
+// a round) H = 20 75.8 / 85.3, H = 60 209 / 235, H = 100 339 / 379; N = 89374 (15 %), H =
+// 60 208.6 / 206.2; N = 108687 (40 %), H = 60 286.1 / 282.9; N = 262143 (37 %), H = 20
+// 169.8 / 181.1; with noise, H = 20, N = 98558 117.0 / 114.4, N = 105275 (35 %)
+// 117.1 / 132.2.  The balance bot, with K in registers, gains from the early start there too
+// (H = 20, N = 450871 43.6 / 42.5).
+inline bool keeps_order(int kind, int lanes, bool k_shared, bool noise, int horizon, long long grid,
+                        long long resident, int warps_per_block, long long tiles, int sms) {
+  const long long warps = resident * warps_per_block;
+  if (tiles > warps) {
+    const long long last = tiles % warps;
+    return kind == kCar && lanes == 1 && k_shared && 10 * last > (noise ? 3 : 2) * warps &&
+           8 * last <= 3 * warps;
+  }
+  if (grid > sms || 2 * grid <= sms || resident <= sms) return false;
+  return horizon >= order_horizon(kind, lanes, k_shared, noise, grid, sms);
+}
+
+}  // namespace mpmi

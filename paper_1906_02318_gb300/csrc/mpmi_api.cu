@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "launch_rules.h"
 #include "tick_dispatch.cuh"
 
 namespace mpmi {
@@ -378,17 +379,11 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
     grid = a.n_units;
   }
   if (grid > s->max_grid[t]) grid = s->max_grid[t];
-  // While the blocks of the tick before hold their SMs, a grid of up to one block per SM
-  // doubles up on the idle ones, and where two blocks on an SM slow each other down more
-  // than the early start gives, the launch keeps the stream's order.  Race car, H = 60, us
-  // in order / early: two lanes, whose warps share K in shared memory, N = 5200 (82
-  // blocks) 35.7 / 41.3, N = 8192 (128) 36.5 / 42.1; eight lanes, K in registers, N = 1500
-  // (94) 20.6 / 18.7, N = 2400 (150) 20.6 / 23.5; sixteen lanes, N = 1024 (128) 18.6 /
-  // 17.7; balance bot, N = 16384 (128) 10.3 / 8.8.  The launches of a screened tick
-  // always follow each other early.
-  const long long sms = s->ctx->sm_count;
-  const bool crowds = k.k_smem > 0 ? 2 * grid > sms : lanes == 8 && 4 * grid > 3 * sms;
-  const bool early = a.chained || !(crowds && grid <= sms && s->max_grid[t] > sms);
+  // the launches of a screened tick always follow each other early
+  const bool early =
+      a.chained || a.n_units > 0 ||
+      !keeps_order(s->model->kind, lanes, k.k_smem > 0, noise, s->cfg.horizon, grid,
+                   s->max_grid[t], block / 32, (n_work + per_warp - 1) / per_warp, s->ctx->sm_count);
   if (a.unit > 0) k.launch_units(a, grid, block, smem + unit_bytes(a.unit), st, early);
   else k.launch(a, grid, block, smem, st, early);
   cudaError_t e = cudaGetLastError();
