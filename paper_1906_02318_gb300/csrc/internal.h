@@ -128,6 +128,7 @@ struct mpmi_ctx {
   uint64_t budget = 0;
   uint64_t used = 0;
   int sm_count = 0;
+  size_t sm_smem = 0;  // shared memory of an SM
   // launch shapes chosen by the autotuner, keyed by (basis, slots, horizon)
   struct TunedShape {
     int kind, n_slots, horizon, lanes, cands, block;
@@ -165,6 +166,7 @@ struct mpmi_session {
   int max_grid[16] = {};
   size_t grid_smem[16] = {};
   int n_units[16] = {};            // the launch kind's sorted units (0: unsorted tiles)
+  bool in_order[16] = {};          // whether it keeps the stream's order (keeps_order)
   mpmi::TickScratch* scratch_dev = nullptr;
   mpmi_result* result_dev = nullptr;
   double* in_dev = nullptr;        // x_t (8 doubles) then u_h (4 doubles)

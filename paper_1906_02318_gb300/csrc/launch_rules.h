@@ -7,6 +7,33 @@
 
 namespace mpmi {
 
+// Whether a one-lane launch over n slots takes sorted units: tiles of per_warp slots, of
+// which one round of the resident warps holds `warps`.  With more than ~1.6 tiles per warp
+// the tiles that a warp saves by sorting outweigh drawing every candidate twice (balance
+// bot, H = 50, N = 65536, 1.7 tiles, 20.8 -> 16.8 us); below, the last round's few tiles
+// run alone either way (race car N = 100000, 1.3 tiles, 217 us unsorted, 225 sorted).  The
+// race car also gains where every tile has a warp of its own (N = 24000 87.7 -> 84.3 us, N
+// = 65536 150 -> 145 us): its warps share the shared-memory pipe, which tiles that leave
+// early free.
+//
+// Short horizons leave little to save.  Balance bot, unsorted / sorted, us: N = 1048576 H
+// = 20 90.6 / 100.0, 30 128.6 / 131.7, 34 143.8 / 140.6, 36 151.3 / 144.5; N = 90396 H = 30
+// 16.5 / 18.8, 36 19.2 / 19.9, 40 19.6 / 20.4, 50 24.0 / 21.6; noisy, N = 1048576 H = 30
+// 392 / 407, 40 498 / 468.  Race car, several rounds: sorting pays there too unless the
+// last round is at most 3/8 full, which unsorted tiles, spread over the SMs, finish sooner
+// (a unit's last tiles go to whichever warps are free, often two on one SM sub-partition):
+// N = 176366 (0.27) H = 20 121.5 / 140.8, 30 175.5 / 202, 40 233 / 262, 44 257 / 277, 52
+// 304 / 308, 60 350 / 332; N = 195473 (0.51) H = 20 144.7 / 141.7; N = 160737 (0.07) H = 20
+// 118.9 / 122.6, 40 229 / 231, 44 252 / 249.
+inline bool units_pay(int kind, int horizon, long long n, int per_warp, long long warps) {
+  const long long wave = warps * per_warp;
+  if (kind != kCar) return horizon >= 35 && 10 * n >= 16 * wave;
+  if (10 * n < 16 * wave) return 2 * n >= wave && n <= wave;
+  if (horizon > 46) return true;
+  const long long last = (n + per_warp - 1) / per_warp % warps;
+  return last == 0 || 8 * last > 3 * warps || (horizon > 32 && 8 * last < warps);
+}
+
 // Horizon from which a tick of S/2 < blocks <= S keeps the stream's order instead of
 // starting early (S: SMs).  While the blocks of the tick before hold their SMs, an early
 // grid doubles up on the idle ones; an early start gives about 2 us whatever the horizon,
@@ -15,7 +42,8 @@ namespace mpmi {
 // where the slower one no longer loses much.  In order / early, us:
 //   race car, K in shared memory (two lanes), 110 blocks: H = 20 16.6 / 14.3, 30 20.7 /
 //     19.5 (79 blocks 18.6 or 24.7), 40 26.2 / 28.3, 60 36.5 / 41.5, 100 53.5 / 64.8;
-//     noisy, 79 to 110 blocks, H = 20 22.7 / 20.5 or 25.0, 30 30.7 / 32.0, 60 53.6 / 60.9
+//     noisy, 79 to 110 blocks, H = 20 22.7 / 20.5 or 25.0, 30 30.7 / 32.0, 60 53.6 / 60.9;
+//     one lane, N = 19000 (149 blocks), H = 20 24.9 / 28.2; four lanes, N = 6000 29.4 / 35.1
 //   eight lanes, 96 blocks: H = 60 20.6 / 18.1, 70 22.7 / 23.0, 100 28.5 / 32.1; noisy, H
 //     = 40 20.6 / 19.3, 60 26.8 / 25.0, 70 30.0 / 32.7; 126 blocks: H = 40 16.6 / 14.3, 60
 //     20.6 / 18.2 or 22.4, 70 22.7 / 23.5; noisy, H = 30 18.6 / 16.2, 40 22.1 / 22.7, 100
@@ -31,12 +59,12 @@ namespace mpmi {
 inline int order_horizon(int kind, int lanes, bool k_shared, bool noise, long long grid, int sms) {
   constexpr int kNever = 1 << 30;
   if (kind == kCar) {
-    if (k_shared) return noise ? 0 : 25;
+    if (k_shared) return noise || lanes != 2 ? 0 : 25;
     if (lanes == 16) return noise ? 55 : 75;
     return 4 * grid > 3LL * sms ? (noise ? 35 : 45) : (noise ? 50 : 65);
   }
   if (kind != kBot || (lanes > 1 && !noise)) return kNever;
-  const int h = lanes > 1 ? 78 : (noise ? 35 : 75);
+  const int h = lanes > 1 ? 78 : (noise ? 35 : 85);
   return 100 * grid > 97LL * sms ? h * 2 / 3 : h;
 }
 
@@ -55,12 +83,18 @@ inline int order_horizon(int kind, int lanes, bool k_shared, bool noise, long lo
 inline bool keeps_order(int kind, int lanes, bool k_shared, bool noise, int horizon, long long grid,
                         long long resident, int warps_per_block, long long tiles, int sms) {
   const long long warps = resident * warps_per_block;
+  if (resident <= sms) return false;  // an SM holds one block: none can double up
   if (tiles > warps) {
     const long long last = tiles % warps;
     return kind == kCar && lanes == 1 && k_shared && 10 * last > (noise ? 3 : 2) * warps &&
            8 * last <= 3 * warps;
   }
-  if (grid > sms || 2 * grid <= sms || resident <= sms) return false;
+  if (2 * grid <= sms) return false;
+  // grids past S blocks: only the race car's one-lane shapes where an SM holds more blocks
+  // than an even spread gives it (blocks of 64 threads, N = 19000, H = 60 65.3 / 75.0; two
+  // candidates per thread, N = 24000, H = 20 35.2 / 31.8)
+  if (grid > sms)
+    return k_shared && lanes == 1 && horizon >= 25 && (grid + sms - 1) / sms < resident / sms;
   return horizon >= order_horizon(kind, lanes, k_shared, noise, grid, sms);
 }
 

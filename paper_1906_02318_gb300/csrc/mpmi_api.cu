@@ -68,35 +68,25 @@ static TickKernel pick_tick(int kind, int lanes, int cands, bool traj, bool nois
 // blocks stage K and the track grid fewer times.
 constexpr int kDefaultBlock = 128;
 
-// Whether a one-lane launch over n slots takes sorted units, where one wave of warps
-// holds `wave` slots.  With more than ~1.6 tiles per warp the tiles a warp saves by
-// sorting outweigh drawing every candidate twice (balance bot N = 65536, 1.7 tiles,
-// 20.8 -> 18.8 us); below, the last round's few tiles run alone either way (race car
-// N = 100000, 1.3 tiles, 217 us unsorted, 225 sorted).  The race car also gains where
-// every tile has a warp of its own (N = 24000 87.7 -> 84.3 us, N = 65536 150 -> 145 us):
-// its warps share the shared-memory pipe, which tiles that leave early free.
-static bool units_pay(int kind, long long n, long long wave) {
-  if (10 * n >= 16 * wave) return true;
-  return kind == kCar && 2 * n >= wave && n <= wave;
-}
-
 // Threads per block the library picks for a shape.  The race car's one-lane
 // shapes: where the warp-tiles fit one block of at most eight warps per SM,
 // blocks of ceil(tiles / SMs) warps, one per SM, load the SMs more evenly than
 // two four-warp blocks on some SMs and one on the rest (measured 4-10 % faster
 // from 20k to 76k slots); everything else kDefaultBlock.
-static int default_block(int kind, int lanes, int cands, long long n_slots, int sms) {
+static int default_block(int kind, int horizon, int lanes, int cands, long long n_slots, int sms) {
   if (lanes == 1) {
     const long long tiles = (n_slots + 32LL * cands - 1) / (32LL * cands);
     const long long w = (tiles + sms - 1) / sms;
     if (kind == kCar && w > 4 && w <= kMaxBlock / 32) return (int)(32 * w);
     // sorted units: one queue of tiles per SM, eight warps on it
-    if (units_pay(kind, n_slots, 256LL * cands * sms) && w > kMaxBlock / 32) return kMaxBlock;
+    if (units_pay(kind, horizon, n_slots, 32 * cands, 8LL * sms) && w > kMaxBlock / 32)
+      return kMaxBlock;
   }
   return kDefaultBlock;
 }
 
-static void default_shape(int kind, int n_slots, int sms, int* lanes, int* cands, int* block) {
+static void default_shape(int kind, int horizon, int n_slots, int sms, int* lanes, int* cands,
+                          int* block) {
   *cands = 1;
   if (kind == kCar) {
     const long long n = n_slots;
@@ -110,7 +100,7 @@ static void default_shape(int kind, int n_slots, int sms, int* lanes, int* cands
   } else {
     *lanes = (kind == kBot && (long long)n_slots * 4 <= (long long)sms * 128) ? 4 : 1;
   }
-  *block = default_block(kind, *lanes, *cands, n_slots, sms);
+  *block = default_block(kind, horizon, *lanes, *cands, n_slots, sms);
 }
 
 TickArgs make_tick_args(const mpmi_session* s, uint64_t tick) {
@@ -337,38 +327,55 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
   const int n_work = (n_hint > 0 && n_hint < s->n_slots) ? n_hint : s->n_slots;
   if (s->max_grid[t] == 0 || s->grid_smem[t] != smem) {
     int nb = 0;
+    const auto plain_blocks = [&]() -> cudaError_t {
+      // static (lane exchange) plus dynamic shared memory may pass the 48 KB default
+      cudaError_t e = smem > 0 ? cudaFuncSetAttribute(
+                                     k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(k.k_smem + kMaxTrackBytes))
+                               : cudaSuccess;
+      if (e != cudaSuccess) return e;
+      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn, block, smem);
+    };
     s->n_units[t] = 0;
     // a grid over one input comes in order as it is (N = 522070, H = 80: 97 us, 109 sorted
     // again)
     const bool ordered = a.sampler == MPMI_SAMPLER_GRID && s->model->nu == 1;
     if (k.fn_units && a.slot_list == nullptr && !ordered) {
       const size_t most = smem + unit_bytes(kUnitMax);
+      int nu = 0;
       cudaError_t e =
           cudaFuncSetAttribute(k.fn_units, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)(k.k_smem + kMaxTrackBytes + unit_bytes(kUnitMax)));
       if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn_units, block, most);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nu, k.fn_units, block, most);
+      // not where the units' buffer costs an SM a block: race car, one candidate per
+      // thread, blocks of 64 threads, N = 50000, H = 60 152 us unsorted, 174 sorted
+      nb = nu;
+      if (e == cudaSuccess && (nu + 1) * most > s->ctx->sm_smem) e = plain_blocks();
       if (e != cudaSuccess) return cuda_fail(e, "sorted units: function attributes");
-      const long long blocks = (long long)nb * s->ctx->sm_count;
-      if (nb > 0 && units_pay(s->model->kind, n_work, blocks * (block / 32) * per_warp)) {
+      const long long blocks = (long long)nu * s->ctx->sm_count;
+      if (nu > 0 && nu >= nb &&
+          units_pay(s->model->kind, s->cfg.horizon, n_work, per_warp, blocks * (block / 32))) {
         // equal shares of the slots per block, in as few rounds as kUnitMax allows
         const long long rounds = (n_work + blocks * kUnitMax - 1) / (blocks * kUnitMax);
         s->n_units[t] = (int)(blocks * rounds);
+        nb = nu;
       }
     }
     if (s->n_units[t] == 0) {
-      // static (lane exchange) plus dynamic shared memory may pass the 48 KB default
-      if (smem > 0) {
-        cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(k.k_smem + kMaxTrackBytes));
-        if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
-      }
-      cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k.fn, block, smem);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+      const cudaError_t e = plain_blocks();
+      if (e != cudaSuccess) return cuda_fail(e, "tick kernel: function attributes");
       if (nb < 1) return fail(MPMI_E_UNSUPPORTED, "tick kernel cannot be resident with this block");
     }
-    s->max_grid[t] = nb * s->ctx->sm_count;
+    const long long blocks = (long long)nb * s->ctx->sm_count;
+    s->max_grid[t] = (int)blocks;
     s->grid_smem[t] = smem;
+    const long long tiles = (n_work + per_warp - 1) / per_warp;
+    s->in_order[t] =
+        s->n_units[t] == 0 &&
+        keeps_order(s->model->kind, lanes, k.k_smem > 0, noise, s->cfg.horizon,
+                    std::min(blocks, (tiles + block / 32 - 1) / (block / 32)), blocks, block / 32,
+                    tiles, s->ctx->sm_count);
   }
   const int per_block = per_warp * (block / 32);
   int grid = (n_work + per_block - 1) / per_block;
@@ -380,10 +387,7 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
   }
   if (grid > s->max_grid[t]) grid = s->max_grid[t];
   // the launches of a screened tick always follow each other early
-  const bool early =
-      a.chained || a.n_units > 0 ||
-      !keeps_order(s->model->kind, lanes, k.k_smem > 0, noise, s->cfg.horizon, grid,
-                   s->max_grid[t], block / 32, (n_work + per_warp - 1) / per_warp, s->ctx->sm_count);
+  const bool early = a.chained || !s->in_order[t];
   if (a.unit > 0) k.launch_units(a, grid, block, smem + unit_bytes(a.unit), st, early);
   else k.launch(a, grid, block, smem, st, early);
   cudaError_t e = cudaGetLastError();
@@ -486,6 +490,7 @@ int mpmi_create(int32_t device, uint64_t mem_budget_bytes, mpmi_ctx** out) {
   c->device = device;
   c->budget = mem_budget_bytes;
   c->sm_count = prop.multiProcessorCount;
+  c->sm_smem = prop.sharedMemPerMultiprocessor;
   *out = c;
   return MPMI_OK;
 }
@@ -780,13 +785,13 @@ int mpmi_session_open(mpmi_ctx* ctx, const mpmi_model* model, const mpmi_session
   if (lanes == 0 && cands > 1) lanes = 1;  // several candidates per thread need one lane
   if (lanes == 0) {
     int dl, dc, db;
-    default_shape(model->kind, (int)slots, ctx->sm_count, &dl, &dc, &db);
+    default_shape(model->kind, cfg->horizon, (int)slots, ctx->sm_count, &dl, &dc, &db);
     lanes = dl;
     if (cands == 0) cands = dc;
   } else {
     if (cands == 0) cands = (lanes == 1 && model->kind == kCar && slots > 48 * 1024) ? 2 : 1;
   }
-  if (block == 0) block = default_block(model->kind, lanes, cands, slots, ctx->sm_count);
+  if (block == 0) block = default_block(model->kind, cfg->horizon, lanes, cands, slots, ctx->sm_count);
   if (block % 32 != 0 || block < 32 || block > kMaxBlock)
     return fail(MPMI_E_INVALID_ARG, "session_open: block must be a multiple of 32 in 32..256");
   if (!pick_tick(model->kind, lanes, cands, false, false).fn)
@@ -1180,7 +1185,7 @@ int mpmi_tune_launch_shape(mpmi_ctx* ctx, const mpmi_model* model,
   if (guard.err != cudaSuccess) return cuda_fail(guard.err, "cudaSetDevice");
   const long long slots = (long long)cfg->n_samples + cfg->include_user;
   int dl = 0, dc = 0, db = 0;
-  default_shape(model->kind, (int)slots, ctx->sm_count, &dl, &dc, &db);
+  default_shape(model->kind, cfg->horizon, (int)slots, ctx->sm_count, &dl, &dc, &db);
   double* in_dev = nullptr;
   mpmi_result* res_dev = nullptr;
   // one start and one end event per timed tick: the ticks are queued back to back

@@ -46,8 +46,7 @@ static bool rounds(long long n) {
 int main() {
   // balance bot
   EXPECT(false, one(kBot, 1, false, 50, 128));
-  EXPECT(true, one(kBot, 1, false, 80, 132));
-  EXPECT(true, one(kBot, 1, false, 50, 152));
+  EXPECT(false, one(kBot, 1, false, 80, 116));
   EXPECT(true, one(kBot, 1, false, 100, 84));
   EXPECT(true, one(kBot, 1, false, 100, 132));
   EXPECT(true, one(kBot, 1, false, 60, 152));
@@ -82,6 +81,37 @@ int main() {
   EXPECT(false, keeps_order(kCar, 1, true, true, 20, 304, 304, 4, (98558 + 63) / 64, 152));
   EXPECT(true, keeps_order(kCar, 1, true, true, 20, 304, 304, 4, (105275 + 63) / 64, 152));
   EXPECT(false, keeps_order(kBot, 1, false, false, 20, 456, 456, 4, 4 * 456 + 600, 152));
+  EXPECT(true, one(kCar, 1, false, 20, 149));
+  EXPECT(true, keeps_order(kCar, 1, true, false, 60, 297, 608, 2, 594, 152));
+  EXPECT(false, keeps_order(kCar, 2, true, false, 60, 257, 304, 4, 1028, 152));
+  EXPECT(false, keeps_order(kCar, 4, true, false, 60, 188, 608, 4, 750, 152));
   // an SM that holds one block has nothing to double up
+  EXPECT(false, keeps_order(kCar, 1, true, false, 60, 152, 152, 8, 1563, 152));
   EXPECT(false, keeps_order(kCar, 2, true, false, 60, 128, 152, 8, 1024, 152));
+""")
+
+
+def test_sorted_units_where_they_pay(tmp_path):
+    _run(tmp_path, r"""
+// balance bot (blocks of 256, one per SM) and race car, two candidates per thread
+static bool bot(int H, long long n) { return units_pay(kBot, H, n, 32, 8 * 152); }
+static bool car(int H, long long n) { return units_pay(kCar, H, n, 64, 8 * 152); }
+int main() {
+  EXPECT(false, bot(20, 1048576));
+  EXPECT(false, bot(30, 1048576));
+  EXPECT(true, bot(36, 1048576));
+  EXPECT(true, bot(50, 65536));
+  EXPECT(false, bot(50, 60000));
+  EXPECT(true, car(60, 65536));
+  EXPECT(true, car(20, 65536));
+  EXPECT(false, car(60, 100000));
+  EXPECT(true, car(60, 176366));
+  EXPECT(false, car(20, 176366));
+  EXPECT(false, car(44, 176366));
+  EXPECT(false, car(20, 262143));
+  EXPECT(true, car(20, 195473));
+  EXPECT(true, car(20, 155648));
+  EXPECT(true, car(44, 160737));
+  EXPECT(false, car(20, 160737));
+  EXPECT(true, units_pay(kCar, 60, 24000, 32, 8 * 152));
 """)
