@@ -98,4 +98,42 @@ inline bool keeps_order(int kind, int lanes, bool k_shared, bool noise, int hori
   return horizon >= order_horizon(kind, lanes, k_shared, noise, grid, sms);
 }
 
+// Which of its other launch shapes an untuned server takes for a batch of that many slots:
+// 0 eight lanes, 1 two lanes, 2 two candidates per thread, -1 the initial one (one lane),
+// for which the batch has `tiles` warp-tiles on `warps` resident warps.
+// Race cars, submit to collect, us.  One session, H = 60: N = 1000 103 -> 65 and N = 3000
+// 103 -> 69 with eight lanes, N = 6000 102 -> 78 and N = 18000 135 -> 99 with two.  Where the
+// one-lane tiles need a second round, two lanes save it (256 slots per SM, seven sessions,
+// 1219 tiles on 1216 warps 190 / 151; three sessions, 1216 tiles 136 / 147; 275 slots per
+// SM, four mixes: 226 / 191 / 185 / 187 -> 176 / 177 / 146 / 173) until theirs is full (420:
+// 209 / 233 / 176 / 225 -> 197 / 227 / 165 / 216).  Past that sessions of one horizon lose
+// (450: 234 / 222 -> 250 / 240; 505: 234 / 228 -> 255 / 245), mixed ones, whose short
+// sessions make room, gain up to 512 (470: 246 / 234 -> 236 / 210; 505: 336 / 213 -> 337 /
+// 202).  Two candidates per thread: see serve_alts.
+inline int serve_alt(int kind, long long slots, long long tiles, long long warps, bool mixed,
+                     int sms) {
+  if (kind != kCar) return -1;
+  if (slots < 32LL * sms) return 0;
+  if (slots < 128LL * sms || (tiles > warps && slots < (mixed ? 512LL : 432LL) * sms)) return 1;
+  return slots >= 1200LL * sms ? 2 : -1;
+}
+
+// Whether a served batch takes sorted units: `horizon` is its longest, `wave` the slots of
+// one tile per resident warp.  A unit costs barriers, and its blocks end the last round
+// together where strided tiles spread it.  Unsorted / sorted, us, submit to collect; the
+// first two of each row mix N and H, the last two are sessions of one N and H = 60:
+//   race cars, one candidate per thread, below two tiles per warp: 93k slots 245 / 274; at
+//     2.15 tiles 289 / 251, 276 / 262, 297 / 322, 279 / 309; 2.3: 307 / 309, 247 / 262, 298
+//     / 326, 286 / 311; 3.1: 401 / 365, 377 / 351, 391 / 414, 373 / 364; 3.9: 418 / 346, 427
+//     / 389, 436 / 435, 416 / 406.  What sorting saves grows with the horizon, so batches
+//     without long ones stay unsorted.
+//   balance bots: 4.1 tiles 117 / 119, 105 / 108, 121 / 135, 102 / 114; 4.5: 96 / 104, 123 /
+//     128, 127 / 138, 103 / 116; 4.7: 116 / 115, 109 / 108, 128 / 130, 106 / 109, one N and
+//     H = 100 131 / 117; 5.1: 99 / 100, 115 / 114, 140 / 134, 116 / 108; 5.9: 128 /
+//     116, 132 / 120, 148 / 139, 123 / 113; H = 30: 7.0 109 / 117, 9.8 136 / 144.
+inline bool serve_units_pay(int kind, int cands, int horizon, long long slots, long long wave) {
+  if (kind == kCar) return slots >= 2 * wave && (cands > 1 || horizon > 64);
+  return horizon >= 35 && 5 * slots >= 23 * wave;
+}
+
 }  // namespace mpmi

@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "launch_rules.h"
 #include "tick_kernel.cuh"
 
 namespace mpmi {
@@ -295,8 +296,7 @@ static std::vector<ServeKernel> serve_shapes(int kind) {
   return {};
 }
 
-// The shapes an untuned server takes instead of the initial one, and which of them
-// (-1: the initial one) a batch of that many slots takes.
+// The shapes an untuned server takes instead of the initial one (serve_alt: which).
 //
 // Large batches: two race cars per thread, so that a word of K from shared memory, which
 // bounds the one-lane step, serves two predictions, in blocks of 256.  Race cars, N and
@@ -306,11 +306,8 @@ static std::vector<ServeKernel> serve_shapes(int kind) {
 // 1853 against 1575.
 //
 // Small race-car batches: several lanes per candidate, as a single tick of that size
-// takes, since one lane's step takes 1.7 us however few there are: one session, H = 60,
-// N = 1000 103 -> 65 us and N = 3000 103 -> 69 with eight lanes, N = 6000 102 -> 78 and N =
-// 18000 135 -> 99 with two.  Two lanes gain again from 256 to 512 slots per SM (277 -> 206,
-// 281 -> 229), but not between (131 -> 136, 176 -> 160, 181 -> 188) nor past it (271 ->
-// 290).  The balance bot gains from neither (four lanes, N = 1000: 46 -> 48).
+// takes, since one lane's step takes 1.7 us however few there are (serve_alt gives the
+// sizes).  The balance bot gains from neither (four lanes, N = 1000: 46 -> 48).
 struct ServeAlt {
   ServeKernel kern;
   int block;
@@ -322,13 +319,6 @@ static std::vector<ServeAlt> serve_alts(int kind) {
             {make_serve<kCar, 1, 2, true>(), 256}};
   return {};
 }
-static int pick_alt(int kind, long long slots, int sms) {
-  if (kind != kCar) return -1;
-  if (slots < 32LL * sms) return 0;
-  if (slots < 128LL * sms || (slots >= 256LL * sms && slots < 512LL * sms)) return 1;
-  return slots >= 1200LL * sms ? 2 : -1;
-}
-
 // Dynamic shared memory of a shape: K and the track grid (a sorted unit on top).
 static size_t serve_smem(const ServeKernel& k, const DevSafety& safety) {
   return k.k_smem + (safety.has_track ? (size_t)safety.track.blob_bytes : 0);
@@ -425,32 +415,38 @@ static int build_graph(mpmi_server* s, ServeShape& shape, int units, int b) {
 }
 
 // Lays out the staged requests: as tiles that the warps stride over, or, where the
-// one-lane shapes have several tiles per warp, as sorted units (sort_unit) that the
-// blocks take from a counter, ordered by horizon, longest first, so that the units
-// taken last are short ones.  Below two tiles per warp the race car loses by a unit's
-// barriers (93k slots 245 -> 274 us), below four the balance bot does (107 us either
-// way).  Mixed sizes and horizons (N log-uniform in 1k..64k, H in 20..100), untuned
-// servers, one candidate per thread, submit to collect: 24 race cars 850 -> 702 us, 60
-// 2320 -> 1860; 24 balance bots 210 -> 168, 60 455 -> 336; both servers together, 48
-// sessions 1077 -> 806 (713 with two race cars per thread).  One to six units per block
-// measured the same within 2 % from two on.
+// one-lane shapes have several tiles per warp (serve_units_pay), as sorted units
+// (sort_unit) that the blocks take from a counter, ordered by horizon, longest first, so
+// that the units taken last are short ones.  Mixed sizes and horizons (N log-uniform in
+// 1k..64k, H in 20..100), untuned servers, one candidate per thread, submit to collect:
+// 24 race cars 850 -> 702 us, 60 2320 -> 1860; 60 balance bots 455 -> 336; both servers
+// together, 48 sessions 1077 -> 806 (713 with two race cars per thread).  One to six
+// units per block measured the same within 2 % from two on.
 // Returns the shape to launch.
 static const ServeShape& plan_batch(const mpmi_server* s, ServeHeader* hdr) {
   SessionTick* ent = reinterpret_cast<SessionTick*>(hdr + 1);
   const int n = hdr->n_requests;
-  long long slots = 0;
-  for (int i = 0; i < n; ++i) slots += ent[i].n_slots;
-  const int alt = pick_alt(s->model->kind, slots, s->ctx->sm_count);
+  const ServeShape& first = s->shape;
+  long long slots = 0, tiles = 0;
+  int horizon = 0, shortest = MPMI_MAX_HORIZON;
+  for (int i = 0; i < n; ++i) {
+    slots += ent[i].n_slots;
+    tiles += (ent[i].n_slots + first.kern.per_warp - 1) / first.kern.per_warp;
+    horizon = std::max(horizon, ent[i].horizon);
+    shortest = std::min(shortest, ent[i].horizon);
+  }
+  const int alt = serve_alt(s->model->kind, slots, tiles,
+                            (long long)first.grid[0] * (first.block / 32),
+                            4 * shortest < 3 * horizon, s->ctx->sm_count);
   const bool other = alt >= 0 && alt < (int)s->alts.size() && s->alts[alt].kern.fn != nullptr;
-  const ServeShape& shape = other ? s->alts[alt] : s->shape;
+  const ServeShape& shape = other ? s->alts[alt] : first;
   const ServeKernel& k = shape.kern;
   std::vector<int> by(n);
   for (int i = 0; i < n; ++i) by[i] = i;
   const int grid = shape.grid[1];  // 0: no sorted units
   const long long warps = (long long)grid * (shape.block / 32);
-  const int min_tiles = s->model->kind == kCar ? 2 : 4;  // per warp
   hdr->unit = 0;
-  if (grid > 0 && slots >= min_tiles * warps * k.per_warp) {
+  if (grid > 0 && serve_units_pay(s->model->kind, k.cands, horizon, slots, warps * k.per_warp)) {
     std::stable_sort(by.begin(), by.end(),
                      [&](int a, int b) { return ent[a].horizon > ent[b].horizon; });
     // a multiple of one tile per warp of a block, about three units per block

@@ -115,3 +115,38 @@ int main() {
   EXPECT(false, car(20, 160737));
   EXPECT(true, units_pay(kCar, 60, 24000, 32, 8 * 152));
 """)
+
+
+def test_served_batches_take_the_faster_shape(tmp_path):
+    _run(tmp_path, r"""
+// one lane per candidate: 32 slots a tile, eight warps an SM; `ragged` more tiles
+static int car(int per_sm, bool mixed = false, int ragged = 0) {
+  return serve_alt(kCar, 152LL * per_sm, 152LL * per_sm / 32 + ragged, 8 * 152, mixed, 152);
+}
+int main() {
+  EXPECT(0, car(20));
+  EXPECT(1, car(100));
+  EXPECT(-1, car(200));
+  EXPECT(-1, car(256));
+  EXPECT(1, car(256, false, 3));
+  EXPECT(1, car(470, true));
+  EXPECT(1, car(505, true));
+  EXPECT(-1, car(520, true));
+  EXPECT(1, car(275));
+  EXPECT(1, car(420));
+  EXPECT(-1, car(450));
+  EXPECT(-1, car(505));
+  EXPECT(-1, car(1000));
+  EXPECT(2, car(1250));
+  EXPECT(-1, serve_alt(kBot, 100, 4, 8 * 152, false, 152));
+  // one tile per warp: 256 slots per SM, a tile of two candidates per thread 512
+  EXPECT(true, serve_units_pay(kCar, 1, 100, 550 * 152, 256 * 152));
+  EXPECT(false, serve_units_pay(kCar, 1, 60, 550 * 152, 256 * 152));
+  EXPECT(false, serve_units_pay(kCar, 1, 60, 800 * 152, 256 * 152));
+  EXPECT(false, serve_units_pay(kCar, 1, 100, 500 * 152, 256 * 152));
+  EXPECT(true, serve_units_pay(kCar, 2, 60, 1250 * 152, 512 * 152));
+  EXPECT(false, serve_units_pay(kBot, 1, 60, 1078 * 152, 256 * 152));
+  EXPECT(false, serve_units_pay(kBot, 1, 60, 1150 * 152, 256 * 152));
+  EXPECT(true, serve_units_pay(kBot, 1, 60, 1250 * 152, 256 * 152));
+  EXPECT(false, serve_units_pay(kBot, 1, 30, 2500 * 152, 256 * 152));
+""")
