@@ -518,10 +518,16 @@ int mpmi_screener_gradients(mpmi_screener* s, const float* features_dev,
                             const float* targets_dev, int32_t batch, float* grad_dev,
                             float* loss_dev, void* stream);
 /* One Adam step (beta1 0.9, beta2 0.999, eps 1e-8) on a minibatch; *loss_dev gets
- * the minibatch loss before the step. */
+ * the minibatch loss before the step.  Should a block's bounded wait for the weights
+ * run out (about two seconds; never expected) the loss comes out NaN and the weights
+ * and Adam's moments stay as they were. */
 int mpmi_screener_train_step(mpmi_screener* s, const float* features_dev,
                              const float* targets_dev, int32_t batch, float lr,
                              float* loss_dev, void* stream);
+/* Test hook, not part of the method: with on != 0 every later gradient or step of the
+ * screener announces the staging of its weights but issues no copy, so that the bounded
+ * wait of its blocks runs out.  on = 0 restores normal training. */
+int mpmi_debug_screener_withhold_staging(mpmi_screener* s, int32_t on);
 /* Network output (sigmoid, predicted ttv / H) for feature rows, computed with
  * bfloat16 weights and activations on tensor cores with float32 accumulation. */
 int mpmi_screener_score(mpmi_screener* s, const float* features_dev, int32_t batch,

@@ -105,7 +105,8 @@ struct TrainSmem {
 template <int SPT>
 __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(const float* P, const float* feats,
                                                                 const float* target, int B,
-                                                                float* part) {
+                                                                float* part, int* late_out,
+                                                                int withhold) {
   using S = TrainSmem<SPT>;
   constexpr int T = S::T;
   extern __shared__ __align__(16) float sm[];
@@ -122,7 +123,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(const float* P, 
   __syncthreads();
   if (tid == 0) bar_expect(&s_bar, kH * kH * 4);
   __syncthreads();
-  if (tid < kH) bulk_g2s(sW2 + tid * kRow, P + oW2 + tid * kH, kH * 4, &s_bar);
+  if (tid < kH && !withhold) bulk_g2s(sW2 + tid * kRow, P + oW2 + tid * kH, kH * 4, &s_bar);
   for (int i = tid; i < kH * kIn; i += kTrainThreads) sW1[i] = P[oW1 + i];
   if (tid < kH) {
     sb1[tid] = P[ob1 + tid];
@@ -333,7 +334,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(const float* P, 
     red[sg] = gb3;
     red[16 + sg] = sq;
   }
-  __syncthreads();
+  const int late = __syncthreads_or(b3 != b3);
+  if (tid == 0) late_out[blockIdx.x] = late;
   if (tid < 2) {
     float v = 0.f;
     for (int i = 0; i < 16; ++i) v += red[16 * tid + i];
@@ -344,28 +346,32 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_tiles(const float* P, 
 // Adds the blocks' records: eight threads per parameter take every eighth record, in
 // order, all of a thread's loads in flight.  With lr > 0 the sum feeds Adam (params, m, v
 // updated in place), else it is stored in grad.  The value after the parameters is the
-// loss.
+// loss.  late[b]: block b's wait for its weights ran out; its record is NaN, and a step
+// leaves the parameters and m, v as they are.
 constexpr int kRedParams = 64, kRedSlices = 8;
 __global__ void __launch_bounds__(kRedSlices * kRedParams)
-    reduce_grad(const float* part, int n_part, int B, float* grad, float* loss, float* P, float* m,
-                float* v, float lr, float c1, float c2) {
+    reduce_grad(const float* part, const int* late, int n_part, int B, float* grad, float* loss,
+                float* P, float* m, float* v, float lr, float c1, float c2) {
   __shared__ float s[kRedSlices][kRedParams];
   const int x = threadIdx.x % kRedParams, y = threadIdx.x / kRedParams;
   const int i = blockIdx.x * kRedParams + x;
   grid_dep_wait();
   grid_dep_release();
+  // a word per thread (there are no more blocks than SMs), in flight with the records
+  int bad = (int)threadIdx.x < n_part ? late[threadIdx.x] : 0;
   float g = 0.f;
   if (i <= kP) {
 #pragma unroll 16
     for (int p = y; p < n_part; p += kRedSlices) g += part[(size_t)p * kPart + i];
   }
   s[y][x] = g;
-  __syncthreads();
+  bad = __syncthreads_or(bad);
   if (y != 0 || i > kP) return;
   g = ((s[0][x] + s[1][x]) + (s[2][x] + s[3][x])) + ((s[4][x] + s[5][x]) + (s[6][x] + s[7][x]));
   if (i == kP) {
     *loss = g / (float)B;
   } else if (lr > 0.f) {
+    if (bad) return;
     const float mi = 0.9f * m[i] + 0.1f * g;
     const float vi = 0.999f * v[i] + 0.001f * g * g;
     m[i] = mi;
@@ -1033,8 +1039,11 @@ struct mpmi_screener {
   float* look = nullptr;
   float half_width = 0.f;
   int max_batch = 0, max_slots = 0;
-  float* part = nullptr;  // n_part gradient records of the training blocks (kPart floats each)
+  // n_part gradient records of the training blocks (kPart floats each), then a word per
+  // block: whether its wait for the weights ran out
+  float* part = nullptr;
   int n_part = 0;
+  int withhold = 0;  // test hook (mpmi_debug_screener_withhold_staging)
   unsigned int* keys = nullptr;
   int* list = nullptr;
   mpmi::ScreenScratch* ss = nullptr;
@@ -1114,17 +1123,18 @@ static int gradients(mpmi_screener* s, const float* feats, const float* target, 
   const int spt = train_spt(B, s->ctx->sm_count);
   const int tiles = (B + 16 * spt - 1) / (16 * spt);
   const int blocks = tiles < s->n_part ? tiles : s->n_part;
+  int* late = reinterpret_cast<int*>(s->part + (size_t)s->n_part * kPart);
   const auto run = [&](auto fn, int smem) {
     return launch_dependent(fn, blocks, kTrainThreads, (size_t)smem, st, (const float*)s->params,
-                            feats, target, B, s->part);
+                            feats, target, B, s->part, late, s->withhold);
   };
   SCR_CUDA(spt == 4   ? run(train_tiles<4>, TrainSmem<4>::BYTES)
            : spt == 2 ? run(train_tiles<2>, TrainSmem<2>::BYTES)
                       : run(train_tiles<1>, TrainSmem<1>::BYTES),
            "train_tiles launch");
   SCR_CUDA(launch_dependent(reduce_grad, (kP + 1 + kRedParams - 1) / kRedParams,
-                            kRedSlices * kRedParams, 0, st, (const float*)s->part, blocks, B, grad,
-                            loss, s->params, s->adam_m, s->adam_v, lr, c1, c2),
+                            kRedSlices * kRedParams, 0, st, (const float*)s->part, (const int*)late,
+                            blocks, B, grad, loss, s->params, s->adam_m, s->adam_v, lr, c1, c2),
            "reduce_grad launch");
   return MPMI_OK;
 }
@@ -1235,8 +1245,9 @@ int mpmi_screener_create(mpmi_ctx* ctx, const mpmi_model* model, const float* we
   std::vector<float> look = lookahead(model->track_host);
   // one record per training block: at most one block per SM, and at most one per 32
   // samples of the largest minibatch
-  s->n_part = (int)std::min<long long>(ctx->sm_count, ((long long)max_batch + 31) / 32);
-  const size_t part_floats = (size_t)s->n_part * kPart;
+  s->n_part = (int)std::min<long long>(std::min(ctx->sm_count, kRedSlices * kRedParams),
+                                       ((long long)max_batch + 31) / 32);
+  const size_t part_floats = (size_t)s->n_part * (kPart + 1);
   const uint64_t bytes = 3 * kP * sizeof(float) + sizeof(InferW) + look.size() * sizeof(float) +
                          part_floats * sizeof(float) +
                          (size_t)max_slots * (sizeof(unsigned int) + sizeof(int)) +
@@ -1356,6 +1367,12 @@ int mpmi_screener_features(mpmi_screener* s, mpmi_session* session, const double
   const int blocks = (session->n_slots + 255) / 256 < 1024 ? (session->n_slots + 255) / 256 : 1024;
   slot_features<<<blocks, 256, 0, (cudaStream_t)stream>>>(a, feature_src(s), out_dev);
   SCR_CUDA(cudaGetLastError(), "slot_features launch");
+  return MPMI_OK;
+}
+
+int mpmi_debug_screener_withhold_staging(mpmi_screener* s, int32_t on) {
+  if (!s) return fail(MPMI_E_INVALID_ARG, "screener is NULL");
+  s->withhold = on ? 1 : 0;
   return MPMI_OK;
 }
 

@@ -96,6 +96,7 @@ _SIGNATURES = {
     "mpmi_server_tune": (c_i32, [c_vp, c_i32, c_vp, c_vp, c_vp, c_i32,
                                  ctypes.POINTER(TuneResult)]),
     "mpmi_debug_withhold_staging": (c_i32, [c_vp, c_i32]),
+    "mpmi_debug_screener_withhold_staging": (c_i32, [c_vp, c_i32]),
     "mpmi_fit_operator_sparse": (c_i32, [ctypes.POINTER(BasisDesc), c_vp, c_vp, c_vp, c_i64,
                                           c_dbl, c_dbl, c_i32, c_vp, c_vp, P_dbl]),
     "mpmi_debug_track_query": (c_i32, [P_dbl, c_i32, c_dbl, c_vp, c_i64, c_vp]),
@@ -682,6 +683,11 @@ class Screener:
         _check(self.ctx.lib.mpmi_screener_train_step(self.handle, _ptr(feats_dev),
                                                      _ptr(targets_dev), feats_dev.shape[0], lr,
                                                      _ptr(loss_dev), _stream(stream)))
+
+    def withhold_staging(self, on: bool):
+        """mpmi_debug_screener_withhold_staging: test hook that makes the training kernel's
+        bounded wait for its weights run out."""
+        _check(self.ctx.lib.mpmi_debug_screener_withhold_staging(self.handle, int(bool(on))))
 
     def score(self, feats_dev, scores_dev, stream=None):
         _check(self.ctx.lib.mpmi_screener_score(self.handle, _ptr(feats_dev), feats_dev.shape[0],

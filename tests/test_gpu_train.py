@@ -56,3 +56,37 @@ def test_gradients_around_the_tiles(setup, B, exact):
         # (2^-24) of the largest entry's terms
         scale = float(np.max(np.abs(ref[k])))
         assert np.max(np.abs(np.asarray(got[k]) - ref[k])) <= 1e-4 * scale + 1e-9, k
+
+
+def test_step_whose_staging_runs_out_keeps_the_weights(setup):
+    """A training step whose weights never arrive in shared memory (test hook): after the
+    bounded wait the loss is NaN, the weights and Adam's moments are untouched, and the
+    following steps are those of a screener that never saw it."""
+    import torch
+    lib, ctx, model = setup
+    rng = np.random.default_rng(5)
+    f = torch.tensor(rng.uniform(-1, 1, (40, 12)), dtype=torch.float32, device="cuda")
+    y = torch.tensor(rng.uniform(0, 1, 40), dtype=torch.float32, device="cuda")
+    loss = torch.zeros(1, device="cuda")
+    out = []
+    for fail in (False, True):
+        scr = lib.Screener(ctx, model, data.screener_init(7), max_batch=64, max_slots=64)
+        losses = []
+        for t in range(3):
+            if fail and t == 1:
+                before = lib.pack_weights(scr.get_weights())
+                scr.withhold_staging(True)
+                scr.train_step(f, y, loss, lr=1e-2)
+                assert np.isnan(float(loss.item()))
+                g = torch.zeros(lib.SCREENER_PARAMS, device="cuda")
+                scr.gradients(f, y, g, loss)
+                assert np.isnan(float(loss.item())) and bool(torch.isnan(g).any())
+                scr.withhold_staging(False)
+                assert np.array_equal(lib.pack_weights(scr.get_weights()), before)
+            scr.train_step(f, y, loss, lr=1e-2)
+            losses.append(float(loss.item()))
+        out.append((losses, lib.pack_weights(scr.get_weights())))
+        scr.free()
+    # the step counter of Adam's bias correction has moved on by the failed step
+    assert out[0][0][:2] == out[1][0][:2]
+    assert np.all(np.isfinite(out[1][1])) and np.max(np.abs(out[0][1] - out[1][1])) < 2e-2
