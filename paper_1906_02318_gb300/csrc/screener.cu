@@ -1243,10 +1243,10 @@ int mpmi_screener_create(mpmi_ctx* ctx, const mpmi_model* model, const float* we
   s->max_slots = max_slots;
   s->half_width = (float)(model->spec.track_half_width - model->spec.inflation);
   std::vector<float> look = lookahead(model->track_host);
-  // one record per training block: at most one block per SM, and at most one per 32
-  // samples of the largest minibatch
+  // one record per training block: at most one block per SM, and one per smallest tile
+  // (train_spt) of the largest minibatch
   s->n_part = (int)std::min<long long>(std::min(ctx->sm_count, kRedSlices * kRedParams),
-                                       ((long long)max_batch + 31) / 32);
+                                       ((long long)max_batch + 15) / 16);
   const size_t part_floats = (size_t)s->n_part * (kPart + 1);
   const uint64_t bytes = 3 * kP * sizeof(float) + sizeof(InferW) + look.size() * sizeof(float) +
                          part_floats * sizeof(float) +

@@ -90,3 +90,17 @@ def test_step_whose_staging_runs_out_keeps_the_weights(setup):
     # the step counter of Adam's bias correction has moved on by the failed step
     assert out[0][0][:2] == out[1][0][:2]
     assert np.all(np.isfinite(out[1][1])) and np.max(np.abs(out[0][1] - out[1][1])) < 2e-2
+
+
+def test_every_smallest_tile_has_a_record(setup):
+    """A screener made for its minibatch can give each tile of 16 samples a block of its
+    own: the records (seen in the memory in use) grow by one per 16 samples."""
+    lib, ctx, model = setup
+    used = []
+    for max_batch in (16, 160, 161):
+        before = ctx.lib.mpmi_memory_in_use(ctx.handle)
+        scr = lib.Screener(ctx, model, data.screener_init(7), max_batch=max_batch, max_slots=64)
+        used.append(ctx.lib.mpmi_memory_in_use(ctx.handle) - before)
+        scr.free()
+    record = 4 * (lib.SCREENER_PARAMS + 1)  # the gradient and the loss
+    assert used[1] - used[0] >= 9 * record and used[2] - used[1] >= record
