@@ -147,11 +147,10 @@ __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_const
   if (fallback_not_needed(a)) return;
   const int n_eval = a.n_list ? *a.n_list : a.n_slots;
   const int H = a.horizon, ro_n = a.ro_n;
-  // equal shares of the candidates, at least one per warp; the blocks that a short
-  // device-side list leaves without a share return at once
+  // the blocks that a short device-side list leaves without a share return at once
   const int wpb = blockDim.x >> 5;
-  const int share = max(wpb, (n_eval + (int)gridDim.x - 1) / (int)gridDim.x);
-  const int n_active = max(1, (n_eval + share - 1) / share);
+  const FactShare in(n_eval, (int)gridDim.x, wpb, (int)blockIdx.x);
+  const int n_active = in.stride;
   if ((int)blockIdx.x >= n_active) {
     if (sure) grid_dep_wait();
     return;
@@ -264,10 +263,7 @@ __global__ void __launch_bounds__(kFactBlock) factored_kernel(const __grid_const
 
   unsigned long long best = ~0ull;
   unsigned int n_safe = 0, n_exec = 0;
-  // the block's candidates, in chunks dealt out in turn (a grid's or a caller's samples
-  // may come in order, and long-lived ones would meet in a few blocks)
-  const UnitSlots in{(int)blockIdx.x, n_active};
-  const int mine = failed ? 0 : unit_count(n_eval, n_active, (int)blockIdx.x);
+  const int mine = failed ? 0 : in.count(n_eval);
   for (int base = 0; base < mine; base += (int)blockDim.x) {
     const int cnt = min((int)blockDim.x, mine - base);
     int slot = 0;
@@ -365,9 +361,9 @@ int launch_factored(mpmi_session* s, TickArgs& a, cudaStream_t st, int n_hint) {
   const size_t track = a.safety.has_track ? (size_t)a.safety.track.blob_bytes : 0;
   const size_t smem = track + (size_t)a.horizon * a.ro_n * sizeof(float4);
   const int n_work = (n_hint > 0 && n_hint < s->n_slots) ? n_hint : s->n_slots;
-  // one candidate per warp until every SM has 32 warps: blocks of 4 to 32 warps
   const int sms = s->ctx->sm_count;
-  const int wpb = std::max(4, std::min(kFactBlock / 32, (n_work + sms - 1) / sms));
+  int wpb, grid;
+  fact_launch(n_work, sms, kFactBlock / 32, &wpb, &grid);
   if (s->fact_grid == 0 || s->fact_smem != smem) {
     if (smem > 0) {
       const size_t cap = kMaxTrackBytes + (size_t)MPMI_MAX_HORIZON * MPMI_MAX_NX * sizeof(float4);
@@ -379,12 +375,9 @@ int launch_factored(mpmi_session* s, TickArgs& a, cudaStream_t st, int n_hint) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, 32 * wpb, smem);
     if (e != cudaSuccess || nb < 1)
       return fail(MPMI_E_UNSUPPORTED, "factored kernel cannot be resident");
-    s->fact_grid = sms;
+    s->fact_grid = sms;  // the check is done
     s->fact_smem = smem;
   }
-  int grid = (n_work + wpb - 1) / wpb;
-  if (grid > s->fact_grid) grid = s->fact_grid;
-  if (grid < 1) grid = 1;
   const cudaError_t e = launch_dependent(fn, grid, 32 * wpb, smem, st, a);
   if (e != cudaSuccess)
     return fail(MPMI_E_CUDA, std::string("factored kernel launch: ") + cudaGetErrorString(e));

@@ -21,6 +21,7 @@
 
 #include <stdint.h>
 
+#include "deal.h"
 #include "internal.h"
 #include "philox.cuh"
 
@@ -709,23 +710,6 @@ __device__ __forceinline__ void fma_word(const float4 kv, const float* z, int w,
   v = __fmaf_rn(kv.y, z[staged_col(KIND, N, 4 * w + 1)], v);
   v = __fmaf_rn(kv.z, z[staged_col(KIND, N, 4 * w + 2)], v);
   v = __fmaf_rn(kv.w, z[staged_col(KIND, N, 4 * w + 3)], v);
-}
-
-// The slots of a sorted unit (see sort_unit): chunks of kUnitChunk consecutive slots,
-// `stride` chunks apart, the first one number `first`.
-constexpr int kUnitChunk = 8;
-struct UnitSlots {
-  int first, stride;
-  __device__ __forceinline__ int slot(int i) const {
-    return (i / kUnitChunk * stride + first) * kUnitChunk + i % kUnitChunk;
-  }
-};
-// Unit u of n_units over n slots: chunks u, u + n_units, ...; its number of slots.
-MPMI_HD int unit_count(int n, int n_units, int u) {
-  const int chunks = (n + kUnitChunk - 1) / kUnitChunk;
-  if (u >= chunks) return 0;
-  const int mine = (chunks - u + n_units - 1) / n_units;
-  return mine * kUnitChunk - ((chunks - 1) % n_units == u ? chunks * kUnitChunk - n : 0);
 }
 
 // One warp-tile: the PER_WARP = 32 C / L candidate positions wt * PER_WARP ...
