@@ -219,8 +219,9 @@ int mpmi_set_safety_set(mpmi_model* model, const mpmi_safety_spec* spec);
 int mpmi_session_open(mpmi_ctx* ctx, const mpmi_model* model,
                       const mpmi_session_config* cfg, mpmi_session** out);
 void mpmi_session_close(mpmi_session* s);
-/* Lanes per candidate, candidates per thread and threads per block the session
- * launches with (any output pointer may be NULL). */
+/* Lanes per candidate, candidates per thread and threads per block that the session's
+ * ticks of the full rollout launch with, its noise taken into account (any output
+ * pointer may be NULL). */
 int mpmi_session_launch_shape(const mpmi_session* s, int32_t* lanes, int32_t* cands,
                               int32_t* block);
 

@@ -276,6 +276,16 @@ int host_tick_end(mpmi_session* s, cudaStream_t st) {
   return MPMI_OK;
 }
 
+// Lanes per candidate of a session's launches over every slot.  Noisy balance-bot ticks of
+// the library's choice: four lanes draw four steps' noise at once, which pays up to 2.5
+// four-lane warps per SM sub-partition (N = 10000 18.5 us against 19.7 with one lane, N =
+// 12000 18.7 against 22.1, N = 16384 23.9 against 23.7).
+static int tick_lanes(const mpmi_session* s) {
+  const bool four = s->n_noise > 0 && s->auto_lanes && s->lanes == 1 && s->model->kind == kBot &&
+                    s->n_slots <= 80 * s->ctx->sm_count;
+  return four ? 4 : s->lanes;
+}
+
 int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, int n_hint,
                      int list_lanes) {
   // a launched tick shares the session's reduction record with the resident kernel
@@ -293,7 +303,7 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamWaitEvent");
     s->tail_pending = false;
   }
-  int lanes = s->lanes, cands = s->cands, block = s->block;
+  int lanes = tick_lanes(s), cands = s->cands, block = s->block;
   // a device-side list short enough that 8 lanes per candidate still fit one wave;
   // n_hint < 0: a list of unknown length (grid for every slot, idle blocks leave)
   const bool small = a.slot_list != nullptr &&
@@ -311,12 +321,6 @@ int launch_tick_args(mpmi_session* s, TickArgs& a, bool traj, cudaStream_t st, i
   }
   if (small) small_shape(s->model->kind, list_lanes, &lanes, &cands, &block);
   const bool noise = a.n_noise > 0;
-  // noisy balance-bot ticks: four lanes draw four steps' noise at once, which pays up to
-  // 2.5 four-lane warps per SM sub-partition (N = 10000 18.5 us against 19.7 with one
-  // lane, N = 12000 18.7 against 22.1, N = 16384 23.9 against 23.7)
-  if (noise && !small && s->auto_lanes && lanes == 1 && s->model->kind == kBot &&
-      s->n_slots <= 80 * s->ctx->sm_count)
-    lanes = 4;
   if (noise && a.tick >= (1ull << 48))
     return fail(MPMI_E_INVALID_ARG, "ticks with noise must stay below 2^48");
   TickKernel k = pick_tick(s->model->kind, lanes, cands, traj, noise);
@@ -891,7 +895,7 @@ void mpmi_session_close(mpmi_session* s) {
 int mpmi_session_launch_shape(const mpmi_session* s, int32_t* lanes, int32_t* cands,
                               int32_t* block) {
   if (!s) return fail(MPMI_E_INVALID_ARG, "session is NULL");
-  if (lanes) *lanes = s->lanes;
+  if (lanes) *lanes = tick_lanes(s);
   if (cands) *cands = s->cands;
   if (block) *block = s->block;
   return MPMI_OK;

@@ -211,3 +211,22 @@ def test_screened_exact_search_with_noise(lib, ctx, car):
                     assert a[key] == b[key], key
                 assert np.array_equal(a["u_r"], b["u_r"])
     scr.free()
+
+
+def test_launch_shape_knows_the_noise(lib, ctx, bot):
+    """The shape a session reports is the one its ticks launch with: noisy balance-bot ticks
+    of few candidates take four lanes where the library chooses, and the caller's lanes
+    otherwise."""
+    env, model = bot
+    s = lib.Session(ctx, model, 10000, 20, env.lo, env.hi)
+    assert s.launch_shape()[0] == 1
+    s.set_noise([0.01] * 4)
+    assert s.launch_shape()[0] == 4
+    s.set_noise([])
+    assert s.launch_shape()[0] == 1
+    s.close()
+    for kw, n, want in ((dict(lanes=1), 10000, 1), (dict(lanes=2), 10000, 2), ({}, 16384, 1)):
+        s = lib.Session(ctx, model, n, 20, env.lo, env.hi, **kw)
+        s.set_noise([0.01] * 4)
+        assert s.launch_shape()[0] == want
+        s.close()
