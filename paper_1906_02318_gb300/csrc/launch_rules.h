@@ -7,6 +7,13 @@
 
 namespace mpmi {
 
+// Candidates per thread of a one-lane launch that leaves them to the library: two race
+// cars past one tile for each of an SM's eight warps (H = 60, one / two, us: N = 39000 134.5
+// / 116.7, 44000 139.8 / 125.3, 48000 143.2 / 128.6).
+inline int one_lane_cands(int kind, long long n, int sms) {
+  return kind == kCar && n > 256LL * sms ? 2 : 1;
+}
+
 // Whether a one-lane launch over n slots takes sorted units: tiles of per_warp slots, of
 // which one round of the resident warps holds `warps`.  With more than ~1.6 tiles per warp
 // the tiles that a warp saves by sorting outweigh drawing every candidate twice (balance

@@ -95,7 +95,7 @@ static void default_shape(int kind, int horizon, int n_slots, int sms, int* lane
     else if (n <= (long long)sms * 128) *lanes = 2;       // two-lane warps fit one wave
     else {
       *lanes = 1;
-      *cands = n > 256LL * sms ? 2 : 1;  // past one tile for each of an SM's eight warps
+      *cands = one_lane_cands(kind, n, sms);
     }
   } else {
     *lanes = (kind == kBot && (long long)n_slots * 4 <= (long long)sms * 128) ? 4 : 1;
@@ -793,7 +793,7 @@ int mpmi_session_open(mpmi_ctx* ctx, const mpmi_model* model, const mpmi_session
     lanes = dl;
     if (cands == 0) cands = dc;
   } else {
-    if (cands == 0) cands = (lanes == 1 && model->kind == kCar && slots > 48 * 1024) ? 2 : 1;
+    if (cands == 0) cands = lanes == 1 ? one_lane_cands(model->kind, slots, ctx->sm_count) : 1;
   }
   if (block == 0) block = default_block(model->kind, cfg->horizon, lanes, cands, slots, ctx->sm_count);
   if (block % 32 != 0 || block < 32 || block > kMaxBlock)

@@ -119,3 +119,19 @@ def test_car_one_lane_default_block_follows_the_sm_count(lib, N, cands):
         assert got["result"][k] == want["result"][k]
     assert np.array_equal(got["result"]["u_r"], want["result"]["u_r"])
     model.free()
+
+
+def test_one_lane_sessions_follow_the_automatic_rule(lib):
+    """A caller who asks for one lane only gets the candidates per thread and the block that
+    the library takes at that size by itself."""
+    ctx = lib.Context(0)
+    env = car_env()
+    model = gpu_model(lib, ctx, env)
+    for n in (30000, 40000, 48000, 70000):
+        shapes = []
+        for kw in ({}, dict(lanes=1)):
+            s = lib.Session(ctx, model, n, 20, env.lo, env.hi, **kw)
+            shapes.append(s.launch_shape())
+            s.close()
+        assert shapes[0] == shapes[1]
+    model.free()

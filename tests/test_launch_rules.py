@@ -150,3 +150,12 @@ int main() {
   EXPECT(true, serve_units_pay(kBot, 1, 60, 1250 * 152, 256 * 152));
   EXPECT(false, serve_units_pay(kBot, 1, 30, 2500 * 152, 256 * 152));
 """)
+
+
+def test_candidates_per_thread_of_one_lane_shapes(tmp_path):
+    _run(tmp_path, r"""
+int main() {
+  EXPECT(1, one_lane_cands(kCar, 38912, 152));
+  EXPECT(2, one_lane_cands(kCar, 39000, 152));
+  EXPECT(1, one_lane_cands(kBot, 1048576, 152));
+""")
