@@ -162,7 +162,8 @@ uint64_t mpmi_memory_in_use(const mpmi_ctx* ctx);
  * x, x_next: m x nx row-major; u: m x nu row-major (the input is held over the
  * step, so the target lifts x_next with the same u).  Solved by Householder QR
  * in float64 on the host, row blocks on several threads (an offline step, Sec. IV-A
- * "learned offline"); the result does not depend on the number of threads.
+ * "learned offline"): at most sixteen, and no more than the CPUs in the calling
+ * thread's affinity mask.  The result does not depend on the number of threads.
  * *residual_out (may be NULL) = ||X K^T - Y||_F / ||Y||_F.  The model's device
  * copy of K is float32 (round to nearest).  Fails with INVALID_ARG when m < n,
  * NONFINITE on NaN/Inf input, and INVALID_ARG if the lifted data is rank

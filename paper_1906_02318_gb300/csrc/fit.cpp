@@ -6,6 +6,7 @@
 // Householder QR of X in float64 (no normal equations, so the conditioning of X
 // is not squared).  The fit runs once per model, offline, on the host.
 #include <math.h>
+#include <sched.h>
 
 #include <algorithm>
 #include <atomic>
@@ -230,12 +231,19 @@ class FitTeam {
   bool stop_ = false;
 };
 
+// CPUs that the calling thread may run on: a caller with a narrower affinity mask (taskset,
+// a container's CPU set, sched_setaffinity) gets no more threads than it has CPUs.
+static int usable_cpus() {
+  cpu_set_t set;
+  if (sched_getaffinity(0, sizeof(set), &set) == 0) return CPU_COUNT(&set);
+  return (int)std::thread::hardware_concurrency();
+}
+
 // Threads for a fit of m rows with p regressors and q targets: one per 8 MFLOP (about
 // a millisecond), at most sixteen.
 static int fit_threads(int64_t m, int p, int q) {
-  const int hw = (int)std::thread::hardware_concurrency();
   const int64_t work = m * p * (p + 2 * q) / 4000000;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(std::min(hw, 16), work));
+  return (int)std::max<int64_t>(1, std::min<int64_t>(std::min(usable_cpus(), 16), work));
 }
 
 // Least squares A W ~= B (A: m x p, B: m x q).  fill(i0, rows, dst): rows [A | B] i0 ..

@@ -55,3 +55,35 @@ def test_same_bits_for_any_thread_count(lib):
                           preexec_fn=lambda c=c: os.sched_setaffinity(0, c)).stdout
            for c in (cpus, cpus[:1])]
     assert out[0] == out[1]
+
+
+def test_threads_stay_within_the_callers_cpus(lib):
+    """A fit starts no more threads than the CPUs that the calling thread may run on, and
+    gives the same bits."""
+    import os
+    import threading
+    import time
+    if not hasattr(os, "sched_setaffinity") or len(os.sched_getaffinity(0)) < 2:
+        pytest.skip("needs two CPUs and an affinity call")
+    x, u, xn = data.transitions("car", 4, 60000)
+    want = lib.fit_operator("car", x, u, xn)
+    out, go = [], threading.Event()
+
+    def fit_on_one_cpu():
+        os.sched_setaffinity(0, {min(os.sched_getaffinity(0))})  # this thread alone
+        go.wait()
+        for _ in range(5):
+            out.append(lib.fit_operator("car", x, u, xn))
+
+    t = threading.Thread(target=fit_on_one_cpu)
+    t.start()
+    time.sleep(0.05)
+    before = most = len(os.listdir("/proc/self/task"))
+    go.set()
+    while t.is_alive():
+        most = max(most, len(os.listdir("/proc/self/task")))
+        time.sleep(0.001)
+    t.join()
+    assert most == before
+    for K, res in out:
+        assert np.array_equal(K, want[0]) and res == want[1]
