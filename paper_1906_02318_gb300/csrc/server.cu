@@ -11,10 +11,10 @@
 // served alone or in a mix.
 //
 // Host side: admission (a free session slot and room in the context's memory
-// budget), kServeBuffers batch buffers, each with a captured graph per launch shape
-// (table upload, kernel, result download) and a stream of its own, so a batch costs one graph
-// launch and up to max_in_flight batches of the model run at once while the
-// requests for the next one are staged.  A session has at most one request
+// budget), kServeBuffers batch buffers, each with a graph (table upload, kernel, result
+// download) and a stream of its own, so a batch costs one graph launch and up to
+// max_in_flight batches of the model run at once while the requests for the next one are
+// staged.  A session has at most one request
 // staged or on the GPU, so batches in flight touch disjoint reduction records;
 // batches are collected in the order they complete.
 #include <cuda_runtime.h>
@@ -248,28 +248,18 @@ __global__ void __launch_bounds__(kMaxBlock, 1) serve_kernel(const __grid_consta
 
 struct ServeKernel {
   const void* fn = nullptr;
-  void (*launch)(const ServeArgs&, int, int, size_t, cudaStream_t) = nullptr;
-  // the same shape over sorted units (one lane)
-  const void* fn_units = nullptr;
-  void (*launch_units)(const ServeArgs&, int, int, size_t, cudaStream_t) = nullptr;
+  const void* fn_units = nullptr;  // the same shape over sorted units (one lane)
   size_t k_smem = 0;
   int per_warp = 32;
   int lanes = 1, cands = 1;
 };
 
-template <int KIND, int L, int C, bool KSMEM, bool UNITS>
-static void launch_serve(const ServeArgs& a, int grid, int block, size_t smem, cudaStream_t st) {
-  serve_kernel<KIND, L, C, KSMEM, UNITS><<<grid, block, smem, st>>>(a);
-}
-
 template <int KIND, int L, int C, bool KSMEM>
 static ServeKernel make_serve() {
   ServeKernel k;
   k.fn = reinterpret_cast<const void*>(&serve_kernel<KIND, L, C, KSMEM, false>);
-  k.launch = &launch_serve<KIND, L, C, KSMEM, false>;
   if constexpr (L == 1) {
     k.fn_units = reinterpret_cast<const void*>(&serve_kernel<KIND, L, C, KSMEM, true>);
-    k.launch_units = &launch_serve<KIND, L, C, KSMEM, true>;
   }
   k.k_smem = (size_t)ksmem_words<KIND, L, KSMEM, true>() * 16;
   k.per_warp = 32 / L * C;
@@ -336,13 +326,24 @@ constexpr int kServeBuffers = 5;                      // batch buffers
 constexpr int kServeMaxInFlight = kServeBuffers - 1;  // one is always free for staging
 
 namespace mpmi {
-// A launch shape of the server with its captured graphs, one per batch buffer, over
-// tiles [0] and over sorted units [1] (one-lane shapes).
+// A launch shape of the server: blocks over tiles [0] and over sorted units [1] (one-lane
+// shapes; 0: none).
 struct ServeShape {
   ServeKernel kern;
   int block = 128;
   int grid[2] = {};
-  cudaGraphExec_t graph[2][kServeBuffers] = {};
+};
+// A batch buffer's graph (table upload, kernel, result download) and what its kernel node
+// launches: the node takes another shape when a batch asks for it (set_launch).  (A graph
+// for every shape, with and without units, was 25 more per race-car server: 3.5 MB of
+// device memory and 0.17 ms of creation; a change of shape costs the next launch about 2.5
+// us.)
+struct ServeGraph {
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  cudaGraphNode_t kernel = nullptr;
+  const void* fn = nullptr;
+  int grid = 0, block = 0;
 };
 }  // namespace mpmi
 
@@ -368,7 +369,7 @@ struct mpmi_server {
   bool flying[kServeBuffers] = {};
   unsigned long long seq[kServeBuffers] = {};  // launch order
   unsigned long long next_seq = 0;
-  cudaStream_t capture = nullptr;
+  mpmi::ServeGraph graph[kServeBuffers];
   int stage = 0;  // buffer receiving requests (never in flight)
   int max_in_flight = kServeMaxInFlight;
   size_t table_bytes = 0;
@@ -388,7 +389,12 @@ static int sfail(cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return sfail(e_, what); \
   } while (0)
 
-static int build_graph(mpmi_server* s, ServeShape& shape, int units, int b) {
+// Gives buffer b's kernel node the shape, over tiles or sorted units, in its graph (under
+// construction: no exec yet) or in the instantiated one.
+static int set_launch(mpmi_server* s, int b, const ServeShape& shape, int units) {
+  ServeGraph& g = s->graph[b];
+  const void* fn = units ? shape.kern.fn_units : shape.kern.fn;
+  if (g.fn == fn && g.grid == shape.grid[units] && g.block == shape.block) return MPMI_OK;
   ServeArgs a;
   memset(&a, 0, sizeof(a));
   a.K = s->model->K32_dev;
@@ -396,21 +402,39 @@ static int build_graph(mpmi_server* s, ServeShape& shape, int units, int b) {
   a.Kp = s->model->K32_dev + 2 * (size_t)s->model->n * s->model->n;
   a.safety = s->model->dev_safety;
   a.table = s->table_dev[b];
-  const size_t smem =
-      serve_smem(shape.kern, s->model->dev_safety) + (units ? unit_bytes(kServeUnit) : 0);
-  cudaGraph_t g = nullptr;
-  SRV_CUDA(cudaStreamBeginCapture(s->capture, cudaStreamCaptureModeThreadLocal), "begin capture");
-  cudaMemcpyAsync(s->table_dev[b], s->table_host[b], s->table_bytes, cudaMemcpyHostToDevice,
-                  s->capture);
-  (units ? shape.kern.launch_units : shape.kern.launch)(a, shape.grid[units], shape.block, smem,
-                                                        s->capture);
-  cudaMemcpyAsync(s->res_host[b], s->res_dev[b], sizeof(mpmi_result) * s->max_sessions,
-                  cudaMemcpyDeviceToHost, s->capture);
-  cudaError_t e = cudaStreamEndCapture(s->capture, &g);
-  if (e != cudaSuccess) return sfail(e, "end capture");
-  e = cudaGraphInstantiate(&shape.graph[units][b], g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) return sfail(e, "graph instantiate");
+  void* args[] = {&a};
+  cudaKernelNodeParams p = {};
+  p.func = const_cast<void*>(fn);
+  p.gridDim = dim3((unsigned)shape.grid[units]);
+  p.blockDim = dim3((unsigned)shape.block);
+  p.sharedMemBytes = (unsigned)(serve_smem(shape.kern, s->model->dev_safety) +
+                                (units ? unit_bytes(kServeUnit) : 0));
+  p.kernelParams = args;
+  const cudaError_t e = g.exec != nullptr
+                            ? cudaGraphExecKernelNodeSetParams(g.exec, g.kernel, &p)
+                            : cudaGraphAddKernelNode(&g.kernel, g.graph, nullptr, 0, &p);
+  if (e != cudaSuccess) return sfail(e, "server graph: kernel node");
+  g.fn = fn;
+  g.grid = shape.grid[units];
+  g.block = shape.block;
+  return MPMI_OK;
+}
+
+static int build_graph(mpmi_server* s, int b) {
+  ServeGraph& g = s->graph[b];
+  SRV_CUDA(cudaGraphCreate(&g.graph, 0), "graph create");
+  const int rc = set_launch(s, b, s->shape, 0);
+  if (rc != MPMI_OK) return rc;
+  cudaGraphNode_t up = nullptr, down = nullptr;
+  SRV_CUDA(cudaGraphAddMemcpyNode1D(&up, g.graph, nullptr, 0, s->table_dev[b], s->table_host[b],
+                                    s->table_bytes, cudaMemcpyHostToDevice),
+           "graph node");
+  SRV_CUDA(cudaGraphAddDependencies(g.graph, &up, &g.kernel, nullptr, 1), "graph dependency");
+  SRV_CUDA(cudaGraphAddMemcpyNode1D(&down, g.graph, &g.kernel, 1, s->res_host[b], s->res_dev[b],
+                                    sizeof(mpmi_result) * s->max_sessions,
+                                    cudaMemcpyDeviceToHost),
+           "graph node");
+  SRV_CUDA(cudaGraphInstantiate(&g.exec, g.graph, 0), "graph instantiate");
   return MPMI_OK;
 }
 
@@ -475,17 +499,11 @@ static int n_flying(const mpmi_server* s) {
   return n;
 }
 
-static void drop_graphs(ServeShape& shape) {
-  for (auto& graphs : shape.graph)
-    for (cudaGraphExec_t& g : graphs) {
-      if (g) cudaGraphExecDestroy(g);
-      g = nullptr;
-    }
-}
-
 static void server_release_device(mpmi_server* s) {
-  drop_graphs(s->shape);
-  for (ServeShape& z : s->alts) drop_graphs(z);
+  for (ServeGraph& g : s->graph) {
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    if (g.graph) cudaGraphDestroy(g.graph);
+  }
   for (int b = 0; b < kServeBuffers; ++b) {
     for (cudaEvent_t e : {s->start[b], s->done[b], s->after[b]})
       if (e) cudaEventDestroy(e);
@@ -496,37 +514,30 @@ static void server_release_device(mpmi_server* s) {
     cudaFree(s->res_dev[b]);
   }
   cudaFree(s->scratch);
-  if (s->capture) cudaStreamDestroy(s->capture);
 }
 
 // Switches a shape record to kernel k with `block` threads per block and a persistent
-// grid (every block resident at once) and captures its batch graphs.  UNSUPPORTED if
-// the shape cannot be resident (the record keeps what it had).
+// grid (every block resident at once).  UNSUPPORTED if the shape cannot be resident (the
+// record keeps what it had).
 static int server_set_shape(mpmi_server* s, ServeShape& shape, const ServeKernel& k, int block) {
   const size_t smem = serve_smem(k, s->model->dev_safety);
   int nb[2] = {};
   for (int units = 0; units < (k.fn_units ? 2 : 1); ++units) {
     const void* fn = units ? k.fn_units : k.fn;
-    const size_t bytes = smem + (units ? unit_bytes(kServeUnit) : 0);
-    if ((bytes > 0 && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)bytes) != cudaSuccess) ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb[units], fn, block, bytes) !=
+    const size_t more = units ? unit_bytes(kServeUnit) : 0;
+    // the largest track's: servers of other models launch the same function
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(k.k_smem + kMaxTrackBytes + more)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb[units], fn, block, smem + more) !=
             cudaSuccess) {
       cudaGetLastError();
       nb[units] = 0;
     }
   }
   if (nb[0] < 1) return fail(MPMI_E_UNSUPPORTED, "server: shape cannot be resident");
-  drop_graphs(shape);
   shape.kern = k;
   shape.block = block;
-  for (int units = 0; units < 2; ++units) {
-    shape.grid[units] = nb[units] * s->ctx->sm_count;
-    for (int b = 0; b < kServeBuffers && shape.grid[units] > 0; ++b) {
-      const int rc = build_graph(s, shape, units, b);
-      if (rc != MPMI_OK) return rc;
-    }
-  }
+  for (int units = 0; units < 2; ++units) shape.grid[units] = nb[units] * s->ctx->sm_count;
   return MPMI_OK;
 }
 
@@ -562,8 +573,7 @@ int mpmi_server_create(mpmi_ctx* ctx, const mpmi_model* model, int32_t max_sessi
     delete s;
     return fail(MPMI_E_OOM, "server: tables exceed the memory budget");
   }
-  bool ok = cudaMalloc(&s->scratch, sizeof(TickScratch) * max_sessions) == cudaSuccess &&
-            cudaStreamCreateWithFlags(&s->capture, cudaStreamNonBlocking) == cudaSuccess;
+  bool ok = cudaMalloc(&s->scratch, sizeof(TickScratch) * max_sessions) == cudaSuccess;
   for (int b = 0; b < kServeBuffers && ok; ++b)
     ok = cudaMallocHost(&s->table_host[b], s->table_bytes) == cudaSuccess &&
          cudaMalloc(&s->table_dev[b], s->table_bytes) == cudaSuccess &&
@@ -595,6 +605,7 @@ int mpmi_server_create(mpmi_ctx* ctx, const mpmi_model* model, int32_t max_sessi
     rc = server_set_shape(s, s->alts.back(), alt.kern, alt.block);
     if (rc == MPMI_E_UNSUPPORTED) rc = MPMI_OK;  // such batches take the initial shape
   }
+  for (int b = 0; b < kServeBuffers && rc == MPMI_OK; ++b) rc = build_graph(s, b);
   if (rc != MPMI_OK) {
     server_release_device(s);
     delete s;
@@ -727,14 +738,15 @@ int mpmi_server_launch(mpmi_server* s, void* stream, int32_t* n_launched) {
     return fail(MPMI_E_NOT_READY, "server_launch: the most batches allowed in flight are on the "
                                   "GPU (collect one first)");
   const ServeShape& shape = plan_batch(s, s->table_host[b]);
+  const int rc = set_launch(s, b, shape, s->table_host[b]->unit ? 1 : 0);
+  if (rc != MPMI_OK) return rc;
   // the batch follows the work queued so far on the caller's stream, and runs
   // on its buffer's own stream so that it overlaps the batches in flight
   cudaStream_t st = (cudaStream_t)stream;
   SRV_CUDA(cudaEventRecord(s->after[b], st), "server event");
   SRV_CUDA(cudaStreamWaitEvent(s->bstream[b], s->after[b], 0), "server stream wait");
   SRV_CUDA(cudaEventRecord(s->start[b], s->bstream[b]), "server event");
-  SRV_CUDA(cudaGraphLaunch(shape.graph[s->table_host[b]->unit ? 1 : 0][b], s->bstream[b]),
-           "server graph launch");
+  SRV_CUDA(cudaGraphLaunch(s->graph[b].exec, s->bstream[b]), "server graph launch");
   SRV_CUDA(cudaEventRecord(s->done[b], s->bstream[b]), "server event");
   if (n_launched) *n_launched = n;
   s->flying[b] = true;
@@ -906,11 +918,7 @@ int mpmi_server_tune(mpmi_server* s, int32_t n, const mpmi_session_config* cfgs,
   // keep the winner (or go back to the initial shape after a failure)
   const int rc2 = server_set_shape(s, s->shape, rc == MPMI_OK ? best_k : initial,
                                    rc == MPMI_OK ? best_block : initial_block);
-  if (rc == MPMI_OK) {  // a tuned server keeps to its winner
-    for (ServeShape& z : alts) drop_graphs(z);
-  } else {
-    s->alts.swap(alts);
-  }
+  if (rc != MPMI_OK) s->alts.swap(alts);  // a tuned server keeps to its winner
   release_all();
   if (rc != MPMI_OK) return rc;
   if (rc2 != MPMI_OK) return rc2;

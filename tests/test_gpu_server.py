@@ -298,3 +298,55 @@ def test_tuned_server_results_equal_alone(lib, ctx, which, n_shapes):
         srv.release(sl)
     srv.free()
     model.free()
+
+
+def test_servers_hold_few_graphs(lib):
+    """A server's graphs are its batch buffers', not one for every launch shape: the device
+    memory that servers of the race car take beside their counted tables."""
+    import torch
+    ctx = lib.Context(0)
+    model = gpu_model(lib, ctx, car_env())
+    servers = [lib.Server(ctx, model, 64)]  # loads the kernels
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    servers += [lib.Server(ctx, model, 64) for _ in range(24)]
+    torch.cuda.synchronize()
+    used = before - torch.cuda.mem_get_info()[0]
+    for s in servers:
+        s.free()
+    model.free()
+    assert used <= 24 * (5 << 20)
+
+
+def test_batches_of_changing_shapes(lib):
+    """Batches that take another launch shape than the one before in the same buffer, with a
+    second server of a smaller track grid beside: each result is that of the tick alone."""
+    ctx = lib.Context(0)
+    env = car_env()
+    model = gpu_model(lib, ctx, env)
+    open_road = lib.model_from_operator(ctx, "car", env.K32)
+    lib.set_safety_set(open_road, env.spec.lo, env.spec.hi)
+    srv, other = lib.Server(ctx, model, 8), lib.Server(ctx, open_road, 2)
+    sizes = [(700, 40), (6000, 30), (20011, 35), (45000, 80), (65536, 90), (65536, 40), (65000, 70)]
+    slots = [srv.admit(n, h, env.lo, env.hi, seed=i) for i, (n, h) in enumerate(sizes)]
+    x = np.tile(data.car_start_state(env.track, vx=12.0), (len(sizes), 1))
+    x[:, 3] += np.arange(len(sizes))
+    u = data.to_f32_exact(np.tile(data.user_input_once(3, env.lo, env.hi), (len(sizes), 1)))
+    # eight lanes, two lanes, one lane, two lanes, units of one and of two candidates per thread
+    batches = [[0], [1], [2], [1, 3], [3, 4], [3, 4, 5, 6], [0], [3, 4, 5, 6], [2], [0], [1]]
+    for t, pick in enumerate(batches):
+        srv.submit([slots[i] for i in pick], x[pick], u[pick], [t] * len(pick))
+        srv.launch()
+        got = dict(srv.collect())
+        for i in pick:
+            n, h = sizes[i]
+            s = lib.Session(ctx, model, n, h, env.lo, env.hi, seed=i, lanes=2)
+            want = run_gpu(lib, s, x[i], u[i], tick=t)["result"]
+            s.close()
+            for k in ("index", "status", "n_safe", "ttv", "cost", "executed_steps"):
+                assert got[slots[i]][k] == want[k], (t, i, k)
+            assert np.array_equal(got[slots[i]]["u_r"], want["u_r"])
+    srv.free()
+    other.free()
+    open_road.free()
+    model.free()
