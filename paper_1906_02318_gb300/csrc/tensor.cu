@@ -134,9 +134,9 @@ __device__ __forceinline__ bool half_any(int h, bool v) {
 
 // LONE: at most one tile per CTA.  Nothing hides the test's chain then, and a lane that
 // tests its own list, four segments at a time, is done sooner than the warp that settles
-// the open positions together, in fewer instructions: H = 60, N = 16384 54.3 -> 51.8 us, N
-// = 38000 60.0 -> 58.7; N = 50000 70.0 against 70.4 the other way.  (An instance of its
-// own: both tests in one kernel cost N = 65536 1.5 %.)
+// the open positions together, in fewer instructions: H = 60, N = 4000 51.7 -> 50.4 us, N
+// = 16384 52.2 -> 50.9, N = 30000 57.7 -> 57.1; N = 50000 70.0 against 70.4 the other way.
+// (An instance of its own: both tests in one kernel cost N = 65536 1.5 %.)
 template <int KIND, bool TRAJ, bool LONE>
 __global__ void __launch_bounds__(kTcThreads, 2) tc_tick_kernel(const __grid_constant__ TickArgs a) {
   using B = BasisTraits<KIND>;

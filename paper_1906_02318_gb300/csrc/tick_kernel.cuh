@@ -14,9 +14,12 @@
 // (double-buffered by step parity, one __syncwarp per step).  L = 1 keeps a
 // whole candidate in one thread; with L = 1 a thread may also carry C
 // candidates, and K may sit in shared memory instead of registers (KSMEM).
-// Warps are persistent: warp w of the grid takes the warp-tiles (32 C / L
-// candidates each) w, w + W, w + 2W, ... so K is loaded once per thread (or
-// block) and the race-car track grid once per block.
+// Warps are persistent, so K is loaded once per thread (or block) and the race-car
+// track grid once per block.  Warp w of the grid takes the warp-tiles (32 C / L
+// candidates each) w, w + W, w + 2W, ...; a large one-lane launch instead gives each
+// block sorted units (sort_unit), whose tiles its warps take from a counter.  The race
+// car's safety test runs beside the next step's product (run_tile, PIPE).  Which launch
+// takes units, and which starts before the kernel in front of it ends: launch_rules.h.
 #pragma once
 
 #include <stdint.h>
@@ -1172,7 +1175,7 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
       advance(t);
       perturb(t);
       record(t);
-    bool any_alive = false;
+      bool any_alive = false;
 #pragma unroll
       for (int c = 0; c < C; ++c) {
         bool ok = box_ok<NX>(safety, z[c]);
@@ -1228,11 +1231,12 @@ __device__ __forceinline__ void run_tile(const P& a, TickDyn d, const DevSafety&
 // chunks from all over the tick: a caller's samples, or a grid's, may come in order, and
 // with a run of them per block the long-lived ones met in a few blocks (balance bot,
 // grid, N = 522070, H = 80: 189 us, 109 in chunks).  A grid over one input needs no
-// sorting at all and takes unsorted tiles (97 us; launch_tick_args).
+// sorting at all and takes unsorted tiles (97 us).
 // GB300, ticks back to back: balance bot H = 50, N = 1048576 207 -> 162 us, H = 100,
 // N = 200000 86 -> 44 us; race car H = 60, N = 65536 150 -> 142 us, N = 262144 578 ->
 // 460 us, H = 100, N = 131072 518 -> 322 us.  Samples already in order of the first
-// input lose what the sorting costs (balance bot, N = 522070, H = 80: 87 -> 92 us).
+// input lose what the sorting costs (balance bot, N = 522070, H = 80: 88.7 -> 91.3 us;
+// random ones 168 -> 92).
 constexpr int kUnitMax = 8192, kUnitBins = 256;
 
 // Shared-memory bytes of a unit: bin counters, each candidate's place and bin.
