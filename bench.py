@@ -28,6 +28,10 @@ test, cost, device-wide argmin and decode (every row of the hot path).
                .. 1048576, one session each: the fraction of the FP32 peak as the
                candidates fill the GPU.
 
+stdout gets one JSON line with the headline, e2e, latency, roofline, clocks and CPU
+baseline; the sections (learned screener, serving, variants, closed loops, roofline_over_n)
+go to stderr, one JSON line each.
+
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 """
 from __future__ import annotations
@@ -1230,11 +1234,27 @@ def main():
         line["roofline_over_n"] = run_over_n(args, out["states"])
     if rank == 0:
         line["cpu_baseline"] = cpu_baseline(args)
-        print(json.dumps(line), flush=True)
+        print_line(line)
     if world > 1:
         import torch.distributed as dist
         dist.barrier()
         dist.destroy_process_group()
+
+
+# Sections beside the headline: long tables, printed to stderr.  With them on it the line on
+# stdout had 20 kB, and a reader that keeps the end of a run's output got half of it.
+SECTIONS = ("learned", "closed_loop_inflated", "serving", "variants", "car_closed_loop",
+            "roofline_over_n", "paper_metrics", "paper_context")
+
+
+def print_line(line: dict) -> None:
+    """The result as one short JSON line on stdout; each section that ran as a JSON line
+    {"section": name, ...} on stderr."""
+    ran = [k for k in SECTIONS if line.get(k) is not None]
+    for k in ran:
+        print(json.dumps({"section": k, k: line[k]}), file=sys.stderr, flush=True)
+    short = {k: v for k, v in line.items() if k not in SECTIONS}
+    print(json.dumps(dict(short, sections_on_stderr=ran)), flush=True)
 
 
 def cpu_baseline(args):
