@@ -61,8 +61,9 @@ inline bool units_pay(int kind, int horizon, long long n, int per_warp, long lon
 //     13.6, 90 12.5 / 13.7, 100 14.4 / 14.9; noisy, H = 30 16.3 / 15.9, 40 18.6 / 19.4, 100
 //     37.0 / 40.9; noisy, four lanes, 124 blocks: H = 70 18.1 / 17.7, 80 18.6 / 19.7, 100
 //     22.7 / 24.3
-// On every SM but a few (152 blocks) the balance bot loses earlier: one lane, H = 50 10.3
-// / 10.4, 60 10.4 / 12.1, 100 14.4 / 17.6.  Its four lanes without noise never do.
+// On every SM or all but one (152 blocks) the balance bot loses earlier: one lane, H = 50
+// 10.3 / 10.4, 60 10.4 / 12.1, 100 14.4 / 17.6 (150 blocks: H = 70 12.4 / 9.5, 90 12.5 /
+// 14.0).  Its four lanes without noise never do.
 inline int order_horizon(int kind, int lanes, bool k_shared, bool noise, long long grid, int sms) {
   constexpr int kNever = 1 << 30;
   if (kind == kCar) {
@@ -72,7 +73,7 @@ inline int order_horizon(int kind, int lanes, bool k_shared, bool noise, long lo
   }
   if (kind != kBot || (lanes > 1 && !noise)) return kNever;
   const int h = lanes > 1 ? 78 : (noise ? 35 : 85);
-  return 100 * grid > 97LL * sms ? h * 2 / 3 : h;
+  return 100 * grid > 99LL * sms ? h * 2 / 3 : h;
 }
 
 // Whether a launch keeps the stream's order: `grid` of at most `resident` blocks with

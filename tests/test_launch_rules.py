@@ -50,6 +50,7 @@ int main() {
   EXPECT(true, one(kBot, 1, false, 100, 84));
   EXPECT(true, one(kBot, 1, false, 100, 132));
   EXPECT(true, one(kBot, 1, false, 60, 152));
+  EXPECT(false, one(kBot, 1, false, 65, 148));
   EXPECT(false, one(kBot, 1, false, 30, 152));
   EXPECT(false, one(kBot, 1, false, 100, 76));
   EXPECT(false, one(kBot, 1, false, 100, 153));
