@@ -26,7 +26,9 @@ inline int one_lane_cands(int kind, long long n, int sms) {
 // Short horizons leave little to save.  Balance bot, unsorted / sorted, us: N = 1048576 H
 // = 20 90.6 / 100.0, 30 128.6 / 131.7, 34 143.8 / 140.6, 36 151.3 / 144.5; N = 90396 H = 30
 // 16.5 / 18.8, 36 19.2 / 19.9, 40 19.6 / 20.4, 50 24.0 / 21.6; noisy, N = 1048576 H = 30
-// 392 / 407, 40 498 / 468.  Race car, several rounds: sorting pays there too unless the
+// 392 / 407, 40 498 / 468.  State by state (40 of them, N = 723704) sorted ticks take 1.01
+// to 1.09 times the unsorted ones at H = 30 (5th to 95th percentile), 0.96 to 1.04 at 34
+// and 0.94 to 1.01 at 36.  Race car, several rounds: sorting pays there too unless the
 // last round is at most 3/8 full, which unsorted tiles, spread over the SMs, finish sooner
 // (a unit's last tiles go to whichever warps are free, often two on one SM sub-partition):
 // N = 176366 (0.27) H = 20 121.5 / 140.8, 30 175.5 / 202, 40 233 / 262, 44 257 / 277, 52
