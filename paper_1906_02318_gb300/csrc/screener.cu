@@ -1243,18 +1243,26 @@ int mpmi_screener_create(mpmi_ctx* ctx, const mpmi_model* model, const float* we
   s->half_width = (float)(model->spec.track_half_width - model->spec.inflation);
   std::vector<float> look = lookahead(model->track_host);
   // one record per training block: at most one block per SM, and one per smallest tile
-  // (train_spt) of the largest minibatch
-  s->n_part = (int)std::min<long long>(std::min(ctx->sm_count, kRedSlices * kRedParams),
-                                       ((long long)max_batch + 15) / 16);
-  const size_t part_floats = (size_t)s->n_part * (kPart + 1);
-  const uint64_t bytes = 3 * kP * sizeof(float) + sizeof(InferW) + look.size() * sizeof(float) +
-                         part_floats * sizeof(float) +
-                         (size_t)max_slots * (sizeof(unsigned int) + sizeof(int)) +
-                         sizeof(ScreenScratch);
-  if (ctx->budget && ctx->used + bytes > ctx->budget) {
-    delete s;
-    return fail(MPMI_E_OOM, "screener exceeds the memory budget");
+  // (train_spt) of the largest minibatch; fewer where the memory budget is short, whose
+  // blocks then take more tiles each
+  constexpr uint64_t kRecord = (kPart + 1) * sizeof(float);
+  const uint64_t rest = 3 * kP * sizeof(float) + sizeof(InferW) + look.size() * sizeof(float) +
+                        (size_t)max_slots * (sizeof(unsigned int) + sizeof(int)) +
+                        sizeof(ScreenScratch);
+  long long records = std::min<long long>(std::min(ctx->sm_count, kRedSlices * kRedParams),
+                                          ((long long)max_batch + 15) / 16);
+  if (ctx->budget) {
+    const uint64_t taken = ctx->used + rest;
+    const uint64_t room = taken < ctx->budget ? (ctx->budget - taken) / kRecord : 0;
+    if (room < 1) {
+      delete s;
+      return fail(MPMI_E_OOM, "screener exceeds the memory budget");
+    }
+    records = std::min<long long>(records, (long long)std::min<uint64_t>(room, 1u << 20));
   }
+  s->n_part = (int)records;
+  const size_t part_floats = (size_t)s->n_part * (kPart + 1);
+  const uint64_t bytes = rest + s->n_part * kRecord;
   bool ok = cudaMalloc(&s->params, kP * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&s->adam_m, kP * sizeof(float)) == cudaSuccess &&
             cudaMalloc(&s->adam_v, kP * sizeof(float)) == cudaSuccess &&

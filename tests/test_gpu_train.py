@@ -104,3 +104,46 @@ def test_every_smallest_tile_has_a_record(setup):
         scr.free()
     record = 4 * (lib.SCREENER_PARAMS + 1)  # the gradient and the loss
     assert used[1] - used[0] >= 9 * record and used[2] - used[1] >= record
+
+
+def test_a_short_budget_takes_fewer_records(setup):
+    """A memory budget that has no room for a record per tile still takes the screener, with
+    fewer records (its blocks loop over tiles), down to one; its gradients meet the same
+    bound.  Below that it is refused."""
+    import torch
+    lib, _, _ = setup
+    record = 4 * (lib.SCREENER_PARAMS + 4)  # the gradient, the loss, padding, the flag
+    free = lib.Context(0)
+    model = gpu_model(lib, free, car_env())
+    base = free.memory_in_use()
+    scr = lib.Screener(free, model, data.screener_init(7), max_batch=320, max_slots=64)
+    whole = free.memory_in_use() - base  # twenty records
+    scr.free()
+    model.free()
+    rng = np.random.default_rng(6)
+    w = data.screener_init(7)
+    f = data.to_f32_exact(rng.uniform(-1, 1, (320, 12)))
+    t = data.to_f32_exact(rng.uniform(0, 1, 320))
+    cache = osc.forward(w, f)
+    ref = osc.backward(w, cache, t)
+    fd = torch.tensor(f, dtype=torch.float32, device="cuda")
+    td = torch.tensor(t, dtype=torch.float32, device="cuda")
+    for fewer in (0, 10, 19):
+        ctx = lib.Context(0, base + whole - fewer * record)
+        model = gpu_model(lib, ctx, car_env())
+        scr = lib.Screener(ctx, model, w, max_batch=320, max_slots=64)
+        assert ctx.memory_in_use() <= base + whole - fewer * record
+        g, loss = torch.zeros(lib.SCREENER_PARAMS, device="cuda"), torch.zeros(1, device="cuda")
+        scr.gradients(fd, td, g, loss)
+        got = lib.unpack_weights(g.cpu().numpy())
+        assert float(loss.item()) == pytest.approx(osc.loss(cache["y"], t), rel=1e-5)
+        for k in ref:
+            scale = float(np.max(np.abs(ref[k])))
+            assert np.max(np.abs(np.asarray(got[k]) - ref[k])) <= 1e-4 * scale + 1e-9, k
+        scr.free()
+        model.free()
+    ctx = lib.Context(0, base + whole - 20 * record)
+    model = gpu_model(lib, ctx, car_env())
+    with pytest.raises(lib.MpmiError):
+        lib.Screener(ctx, model, w, max_batch=320, max_slots=64)
+    model.free()
